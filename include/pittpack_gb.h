@@ -82,17 +82,17 @@ typedef struct pp_plan_options {
   int threads_y_inv;
   int cols_y_inv;
   int z_method;    /* periodic z only: 0 = automatic (Sherman-Morrison, or with autotune = 1 the
-                      faster of the two, timed), 1 = Sherman-Morrison sweeps, 2 = DFT along z and a
+                      faster of the two, timed), 1 = Sherman-Morrison, 2 = DFT along z and a
                       diagonal solve (needs nz = 2^a 3^b 5^c 7^d <= 4096, else
                       PP_ERR_UNSUPPORTED_SIZE); ignored for non-periodic z */
-  int z_split;     /* non-periodic z only: 0 = automatic (the Thomas sweeps, or with autotune = 1
-                      the fastest of them and the partitioned solves, timed as a lone launch),
+  int z_split;     /* non-periodic z only: 0 = automatic (by the grid's size, or with autotune = 1
+                      the fastest of the sweeps and the partitioned solves, timed as a lone launch),
                       1 = Thomas sweeps, 8 / 16 / 32 = partitioned solve: every z line split into
                       chunks of that many rows, one thread per chunk, the chunk carries combined by
-                      recursive doubling (log2 of the chunk count levels; see pp_plan_z_split).
-                      Needs nz <= 512 x rows (else PP_ERR_UNSUPPORTED_SIZE); other values
-                      PP_ERR_INVALID_ARG; ignored for periodic z and for the adjoint's transposed
-                      solve, which run the sweeps */
+                      a short sum or recursive doubling (see pp_plan_z_split).  Needs
+                      nz <= 512 x rows (else PP_ERR_UNSUPPORTED_SIZE); other values
+                      PP_ERR_INVALID_ARG; ignored for periodic z, whose Sherman-Morrison solve
+                      always takes the automatic choice */
   int reserved[1]; /* must be zero */
 } pp_plan_options;
 
@@ -185,7 +185,7 @@ pp_status pp_fold_bc(pp_plan* plan, const void* f_in, void* f_out, const void* c
  * against 4.30 ms FP64).  So the first call over a list of plans that includes autotuned members
  * waits for `stream` to be idle, allocates scratch grids of the members' sizes for the duration
  * of the call, and times the graph with the members' own settings and with the default launch
- * shapes and z sweeps (Thomas; Sherman-Morrison for periodic z) for the autotuned members; the
+ * shapes and the automatic z solve (z_split = 0, z_method = 0) for the autotuned members; the
  * faster is kept for that list of plans (the plans themselves keep their settings for pp_solve).
  * Without the scratch memory, or while `stream` is being captured into a graph, the members' own
  * settings are used.
@@ -197,7 +197,8 @@ pp_status pp_solve_batched(pp_plan* const* plans, const void* const* f, void* co
 /* Adjoint: g_f = S^T g, where S is the solution operator f -> u.  Runs the transposed
  * pipeline: the line transforms, whose unnormalised syntheses are the transposes of the analyses
  * up to the per-mode weights the z scale absorbs, around the transposed tridiagonal
- * factorisation (for non-periodic z).  For periodic z the Sherman-Morrison sweep is run as it is
+ * factorisation (non-periodic z; the partitioned solve of FP64-class plans runs as it is, the
+ * row-scaled tridiagonal matrix being symmetric).  For periodic z the Sherman-Morrison sweep is run as it is
  * (A' and its rank-one update are symmetric, so that solve is its own transpose), and so is the
  * z transform (its eigenvalues are even in kz).  A is symmetric for periodic, Neumann and
  * Dirichlet faces, so S^T = S.  Same argument rules as pp_solve. */
@@ -258,10 +259,12 @@ pp_status pp_plan_z_method(const pp_plan* plan, int* out);
  * partitioned solve (Sec. "Solution of the Resulting Tridiagonal Matrices", with the sequential
  * sweep replaced as in the parallel alternatives of Sec. "Cyclic Reduction Technique"): each line
  * is cut into ceil(nz / M) chunks of M rows, every chunk runs both recurrences of the Thomas
- * factorisation from a zero carry, and the chunks' affine carry maps are combined by recursive
- * doubling, ceil(log2(nz / M)) levels.  Same multipliers and results as the sweeps up to rounding;
- * about three times their arithmetic per value, in exchange for nz / M times the threads.  Chosen
- * by options.z_split or the autotuner; periodic z reports 1.  Errors: PP_ERR_INVALID_ARG (NULL). */
+ * factorisation from a zero carry for the value that leaves it and again from its true carry, which
+ * comes from the chunks nearby (a mode decays along its line) or, for weakly dominant modes, from
+ * recursive doubling over ceil(log2(nz / M)) levels.  Same multipliers and results as the sweeps up
+ * to rounding; about half again their arithmetic, in exchange for nz / M times the threads.  Chosen
+ * by options.z_split, by the grid's size or by the autotuner; periodic z reports 1.  Errors:
+ * PP_ERR_INVALID_ARG (NULL). */
 pp_status pp_plan_z_split(const pp_plan* plan, int* out);
 
 /* ---- Prototype, not used by the solver: a DFT stage on the tensor cores (tcgen05, TMEM). ----

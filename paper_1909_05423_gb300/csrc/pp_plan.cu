@@ -32,7 +32,7 @@ namespace pp {
 cudaError_t launch_lines_impl(const LineArgs& a, bool df_arith, int oy, int sin, int sout, int threads,
                               cudaStream_t st);
 cudaError_t launch_zsolve_impl(const ZArgs& a, bool df_spill, bool zper, cudaStream_t st);
-cudaError_t launch_zpart_impl(const ZArgs& a, bool df_spill, int M, cudaStream_t st);
+cudaError_t launch_zpart_impl(const ZArgs& a, bool df_spill, bool zper, int M, cudaStream_t st);
 cudaError_t launch_zdiag_impl(const ZDiagArgs& a, bool df_spill, cudaStream_t st);
 }  // namespace pp
 
@@ -668,6 +668,7 @@ static void zsolve_args(const pp_plan* p, void* data, int transpose, ZArgs& a) {
   a.qtab = p->d_qtab;
   split2(p->zscale, a.scale);
   a.transpose = transpose;
+  a.nsing = p->singular ? (a.cplx ? 2 : 1) : 0;
   a.rstat = p->d_status;
   a.dmin = 0x1p-100f;
   a.umax = (float)(0x1p124 / ((double)p->nx * (double)p->ny));
@@ -680,21 +681,12 @@ cudaError_t launch_zsolve(const pp_plan* p, void* data, int transpose, cudaStrea
   ZArgs a;
   zsolve_args(p, data, transpose, a);
   const bool zper = p->bc[4] == PP_BC_PERIODIC;
-  // the partitioned solve runs the forward factorisation of non-periodic z (the transposed one of
-  // the adjoint stays on the Thomas sweeps); it leaves the singular mode to the pinned sweep
-  if (p->zsplit > 1 && !zper && !transpose) {
-    cudaError_t e = launch_zpart_impl(a, p->dtype == PP_F64, p->zsplit, st);
-    if (e != cudaSuccess || !p->singular) return e;
-    return launch_zsingular(p, data, st);
-  }
+  // The partitioned solve serves the adjoint of FP64-class plans as it is: the row-scaled matrix is
+  // symmetric, so its transposed system is the same one.  Mixed plans keep the transposed sweeps, whose
+  // roundings to the FP32 spill fall on other values than the forward factorisation's.
+  const bool tr32 = transpose && !zper && p->dtype != PP_F64;
+  if (p->zsplit > 1 && !tr32) return launch_zpart_impl(a, p->dtype == PP_F64, zper, p->zsplit, st);
   return launch_zsolve_impl(a, p->dtype == PP_F64, zper, st);
-}
-
-cudaError_t launch_zsingular(const pp_plan* p, void* data, cudaStream_t st) {
-  ZArgs a;
-  zsolve_args(p, data, 0, a);
-  a.only_singular = 1;
-  return launch_zsolve_impl(a, p->dtype == PP_F64, false, st);
 }
 
 // z lines as strided columns: the y-orientation kernels with one "plane" of splane/2 complex columns
@@ -782,6 +774,30 @@ static pp_status run_stage(pp_plan* p, int stage, const void* f, void* u, int tr
   }
   if (e != cudaSuccess) return fail(PP_ERR_CUDA, "%s launch: %s", names[stage], cudaGetErrorString(e));
   return PP_OK;
+}
+
+// Rows per chunk of the z solve when nobody chose them (1: the sweeps), by what was measured (GB300, z
+// stage alone; sweeps / 8 rows / 16 rows, ms):
+//   FP64   32^3 0.028/0.011/0.013   128^3 0.122/0.022/0.026   256^3 0.309/0.113/0.104
+//          256 x 384^2 0.379/0.248/0.225   256 x 512^2 0.471/0.432/0.387   1024 x 512^2 1.63/2.05/1.64
+//          1024^3 4.32/8.2/6.5   4095 x 64^2 3.37/0.197/0.180
+//          periodic z: 192^3 0.246/0.076/0.082   512^3 1.162/1.126/1.163
+//   mixed  256 x 320^2 0.240/0.156/0.137   256 x 448^2 0.299/0.301/0.262   64 x 512^2 0.092/0.113/0.105
+//          512^3 0.61/0.83/0.67   periodic z: 256^3 0.274/0.133/0.145
+// The sweeps read and write at the copy bandwidth once their threads (one per real slot) fill the GPU;
+// below that a line's serial chain sets their time, whatever the number of lines.  The partitioned solve
+// does 1.5 times their arithmetic and takes 6 ps a value.  The lines cross near 290 k slots for the
+// double-float spill (checkpointed sweeps) and 230 k for FP32.  16 rows a chunk do less carry work, 8
+// give twice the threads: worth it up to 8 M values, and for periodic z, whose q terms weigh on the
+// first chunks.
+static int z_rows_default(const pp_plan* p) {
+  const bool zper = p->bc[4] == PP_BC_PERIODIC;
+  if (p->splane > (p->dtype == PP_F64 ? 290000 : 230000)) return 1;
+  int M = (zper || p->splane * p->nz <= (8LL << 20)) ? 8 : 16;
+  int G, lgG, P;
+  for (; M <= 32; M *= 2)
+    if (zpart_shape(p->nz, M, (int)p->elem, &G, &lgG, &P)) return M;
+  return 1;
 }
 
 static pp_status run_pipeline(pp_plan* p, const void* f, void* u, int transpose, cudaStream_t st, int io = -1,
@@ -962,31 +978,25 @@ static pp_status autotune(pp_plan* p, bool zmethod_free, bool zsplit_free) {
     if (run_stage(p, stage, f, u, 0, st) != PP_OK) break;  // leave this stage's output for the next one
   }
   const float bx = std::max(bt[0], bt[3]), by = std::max(bt[1], bt[2]);
-  // periodic z: Sherman-Morrison sweeps or the z transform, unless the caller chose one
-  int zbest = p->zmethod;
-  if (p->zfft_ok && zmethod_free) {
-    float tz[2];
-    for (int m = 0; m < 2; m++) {
-      p->zmethod = m;
-      tz[m] = time_stage(2);
-    }
-    zbest = (tz[ZM_FFT] < tz[ZM_SM]) ? ZM_FFT : ZM_SM;
-  }
-  p->zmethod = zbest;
-  // non-periodic z: the Thomas sweeps or the partitioned solve with 8 / 16 / 32 rows per chunk,
-  // timed as a lone launch (the partitioned solve trades extra arithmetic for parallelism, which
-  // pays when a plan has too few modes to fill the GPU)
-  if (zsplit_free && p->bc[4] != PP_BC_PERIODIC) {
+  // the sweeps (Thomas or Sherman-Morrison) or the partitioned solve with 8 / 16 / 32 rows per chunk,
+  // timed as a lone launch (the partitioned solve trades extra arithmetic for parallelism, which pays
+  // when a plan has too few modes to fill the GPU)
+  float tsm = 1e30f;
+  if (zsplit_free && p->zmethod == ZM_SM) {
     int sbest = 1;
-    float tbest = 1e30f;
     for (int M : {1, kZSplitRows[0], kZSplitRows[1], kZSplitRows[2]}) {
       int G, lgG, P;
-      if (M > 1 && !zpart_shape(p->nz, M, &G, &lgG, &P)) continue;
+      if (M > 1 && !zpart_shape(p->nz, M, (int)p->elem, &G, &lgG, &P)) continue;
       p->zsplit = M;
       const float t = time_stage(2);
-      if (t < tbest) { tbest = t; sbest = M; }
+      if (t < tsm) { tsm = t; sbest = M; }
     }
     p->zsplit = sbest;
+  }
+  // periodic z: those or the z transform, unless the caller chose one
+  if (p->zfft_ok && zmethod_free) {
+    p->zmethod = ZM_FFT;
+    if (time_stage(2) >= tsm) p->zmethod = ZM_SM;
   }
   cudaStreamSynchronize(st);
   for (int i = 0; i < kTuneStreams; i++) {
@@ -1082,9 +1092,8 @@ static void set_settings(pp_plan* p, const PlanSettings& s) {
 }
 
 // Puts the autotuned members of a batch on the library's shared-GPU settings -- the default launch
-// shapes and, where the autotuner chose the z algorithm, the Thomas or Sherman-Morrison sweeps
-// (the partitioned solve and the z transform buy a lone plan latency with extra work) -- for the
-// scope of one capture, and restores their own settings afterwards (a captured graph keeps the
+// shapes and, where the autotuner chose the z algorithm, the default one of its size (the z transform
+// buys a lone plan latency with extra work) -- for the scope of one capture, and restores their own settings afterwards (a captured graph keeps the
 // launch parameters it was captured with).
 struct SettingsSwap {
   std::vector<std::pair<pp_plan*, PlanSettings>> saved;
@@ -1098,7 +1107,7 @@ struct SettingsSwap {
       saved.emplace_back(p, get_settings(p));
       choose_shapes(p, nullptr);
       if (p->z_tuned) {
-        p->zsplit = 1;
+        p->zsplit = z_rows_default(p);
         p->zmethod = ZM_SM;
       }
     }
@@ -1287,7 +1296,7 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   const int sreq = (opt && !zper) ? opt->z_split : 0;
   if (sreq > 1) {
     int G, lgG, P;
-    if (!zpart_shape(nz, sreq, &G, &lgG, &P))
+    if (!zpart_shape(nz, sreq, dtype == PP_F64 ? 8 : 4, &G, &lgG, &P))
       return fail(PP_ERR_UNSUPPORTED_SIZE, "z_split %d: nz = %d needs more than 512 chunks per line", sreq, nz);
   }
 
@@ -1319,7 +1328,7 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   p->zfft_ok = zfft_ok;
   if (p->zfft_ok && (s = zfft_tables(p)) != PP_OK) { free_plan(p); return s; }
   p->zmethod = (zreq == 2) ? ZM_FFT : ZM_SM;
-  p->zsplit = (sreq > 1) ? sreq : 1;
+  p->zsplit = sreq ? sreq : z_rows_default(p);
   choose_shapes(p, opt);
 
   p->buf_bytes = (size_t)std::max(p->xplane, p->splane) * nz * p->elem;
@@ -1333,10 +1342,10 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   }
   cudaMemset(p->d_status, 0, 4 * sizeof(unsigned));
   if (opt && opt->autotune) {
-    pp_status ts = autotune(p, zreq == 0, sreq == 0 && !zper);
+    pp_status ts = autotune(p, zreq == 0, sreq == 0);
     if (ts != PP_OK) { free_plan(p); return ts; }
     p->tuned = true;
-    p->z_tuned = zper ? (zreq == 0 && zfft_ok) : (sreq == 0);
+    p->z_tuned = zper ? (zreq != 2) : (sreq == 0);
   }
   *out = p;
   return PP_OK;

@@ -19,31 +19,24 @@ namespace pp {
 __device__ __forceinline__ void track(float& m, float v) {
   asm("max.NaN.f32 %0, %0, %1;" : "+f"(m) : "f"(fabsf(v)));
 }
-__device__ __forceinline__ float max_nan(float a, float b) {
-  float r;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
 
 // Block reduction of the two maxima (blocks of at most 1024 threads, every thread calls it) and
 // the per-launch decision of the last block.  rstat: [0] status bits, [1] / [2] running maxima
 // (FP32 bits), [3] count of finished blocks; nblocks: blocks of the launch.
 __device__ __forceinline__ void range_report(unsigned* rstat, float dmin, float umax_lim, unsigned nblocks,
                                              float dmax, float umax) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dmax = max_nan(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-    umax = max_nan(umax, __shfl_xor_sync(0xffffffffu, umax, o));
-  }
-  __shared__ float s_d[32], s_u[32];
-  const int w = (int)threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { s_d[w] = dmax; s_u[w] = umax; }
+  // non-negative floats and NaN order as their bit patterns (sign cleared), so one warp reduction of the
+  // bits serves each maximum
+  __shared__ unsigned s_d[32], s_u[32];
+  const unsigned dw = __reduce_max_sync(0xffffffffu, __float_as_uint(dmax) & 0x7fffffffu);
+  const unsigned uw = __reduce_max_sync(0xffffffffu, __float_as_uint(umax) & 0x7fffffffu);
+  const int w = (int)threadIdx.x >> 5, nw = ((int)blockDim.x + 31) >> 5;
+  if ((threadIdx.x & 31) == 0) { s_d[w] = dw; s_u[w] = uw; }
   __syncthreads();
+  if (w != 0) return;
+  const unsigned db = __reduce_max_sync(0xffffffffu, (int)threadIdx.x < nw ? s_d[threadIdx.x] : 0u);
+  const unsigned ub = __reduce_max_sync(0xffffffffu, (int)threadIdx.x < nw ? s_u[threadIdx.x] : 0u);
   if (threadIdx.x != 0) return;
-  float D = s_d[0], U = s_u[0];
-  for (int i = 1; i < ((int)blockDim.x + 31) / 32; i++) { D = max_nan(D, s_d[i]); U = max_nan(U, s_u[i]); }
-  // non-negative floats and NaN order as their bit patterns (sign cleared)
-  const unsigned db = __float_as_uint(D) & 0x7fffffffu, ub = __float_as_uint(U) & 0x7fffffffu;
   unsigned* r = rstat;
   if (db > *reinterpret_cast<volatile unsigned*>(r + 1)) atomicMax(r + 1, db);
   if (ub > *reinterpret_cast<volatile unsigned*>(r + 2)) atomicMax(r + 2, ub);

@@ -1,4 +1,4 @@
-// pp_zpart.cu -- the z tridiagonal solve of non-periodic z with every line split into chunks
+// pp_zpart.cu -- the z tridiagonal solve with every line split into chunks
 // (Sec. "Solution of the Resulting Tridiagonal Matrices"; the parallel alternatives to the
 // sequential Thomas sweep of Sec. "Cyclic Reduction Technique" / "Parallel Cyclic Reduction").
 //
@@ -6,31 +6,44 @@
 // with the plan's precomputed multipliers w_k:
 //     forward   g_k = (s d_k - g_{k-1}) w_k = a_k g_{k-1} + w_k s d_k,      a_k = -w_k, g_{-1} = 0,
 //     backward  u_k = g_k - w_k u_{k+1}     = a_k u_{k+1} + g_k,            u_n = 0.
-// One thread per line runs them in sequence: with few modes and long lines (the setting of the
-// paper's solver comparison, 64 x 64 modes and up to 4095 rows) the GPU has too few threads for
-// that.  Here a line is split into P chunks of M consecutive rows, one thread per chunk, and each
-// recurrence is solved in three steps:
-//   1. every thread runs the recurrence over its chunk from a zero carry, keeping the local
-//      values and the chunk's affine map x_out = A x_in + B (A the product of its a_k);
-//   2. the maps of the P chunks of a line are composed by recursive doubling (Kogge-Stone: at
-//      level j every chunk composes its map with the one 2^j chunks before it), with warp
-//      shuffles inside a warp's run of chunks and one shared-memory exchange of the warps' totals,
-//      which gives each chunk its true carry;
-//   3. every thread adds (product of a_i up to row k) x carry to its local values.
-// The multipliers and the order of the per-row operations are those of the Thomas sweeps, so the
-// result is the Thomas result up to the rounding of the chunk products; unlike cyclic reduction
-// applied to the rows of the tridiagonal system, nothing forms the reduced systems' diagonals,
-// whose distance from weak diagonal dominance (about the square of the lowest wavenumber)
+// One thread per line runs them in sequence, and reads every value twice: with fewer than about
+// 150 k lines the GPU has too few threads for that, and a 256-row chain of double-float steps takes
+// 0.3 ms however few lines there are.  Here a line is split into P chunks of M consecutive rows, one
+// thread per chunk, whose M values stay in registers from the one load to the one store.  Each
+// recurrence runs twice over them:
+//   1. from a zero carry, only to get B, the value that leaves the chunk; the value that enters it
+//      adds A x_in with A the product of the chunk's a_k;
+//   2. from the chunk's true carry, keeping the values.
+// A second run of the recurrence costs less than adding (product of a_i up to row k) x carry to the
+// kept values of the first (which the products alone make 1.5 times as long), and its rounding is that
+// of the plain sweep.
+// The carry of chunk c is B_{c-1} + A_{c-1} (B_{c-2} + A_{c-2} (...)).  A decays by the mode's
+// multiplier to the power M, so for most modes a few terms reach 2^-56 of the first and every thread
+// sums them itself (Horner, at most kZpWindow terms); a CTA that holds a slower mode composes the
+// chunk maps by recursive doubling instead, with warp shuffles inside a warp's run of chunks and one
+// shared-memory exchange of the warps' totals.
+// The multipliers and the order of the per-row operations are those of the Thomas sweeps; unlike
+// cyclic reduction applied to the rows of the tridiagonal system, nothing forms the reduced systems'
+// diagonals, whose distance from weak diagonal dominance (about the square of the lowest wavenumber)
 // double-float coefficients would not keep.
 //
-// The M values of a thread stay in registers between the steps.  A CTA takes G adjacent real slots (consecutive threads: consecutive slots, so
-// every row access of a warp is a few contiguous segments) x P chunks; G P <= 512.  Padding slots
-// take part in the scans with their maps unused; the singular mode's column is left untouched
-// (the plan solves it with the pinned Thomas sweep afterwards).
+// Periodic z is the Sherman-Morrison form of pp_zsolve.cu: the partial sums of y_0 = sum q_k d_k
+// travel with the forward carries, the last chunk's thread forms c, and the back substitution starts
+// from u_n = c.  The adjoint's transposed system is the same one (the row-scaled matrix is symmetric;
+// FP64-class plans run it here).
 //
-// Arithmetic: double-float (pp_arith.cuh) on the plan's spill type.  Range report: pp_range.cuh.
+// A CTA takes G adjacent real slots (consecutive threads: consecutive slots, so every row access of a
+// warp is a few contiguous segments) x P chunks.  The singular mode's slots are solved by one more CTA
+// each (pp_zsing.cuh).
+//
+// Arithmetic: double-float (pp_arith.cuh) on the plan's spill type, normalised steps for the
+// double-float spill and unnormalised ones for FP32 (as in the sweeps).  Range report: pp_range.cuh.
+#include <algorithm>
+#include <atomic>
+
 #include "pp_range.cuh"
 #include "pp_zmul.cuh"
+#include "pp_zsing.cuh"
 
 namespace pp {
 
@@ -40,9 +53,6 @@ __device__ __forceinline__ void zp_st(float2* p, df v) { *p = make_float2(v.hi, 
 __device__ __forceinline__ void zp_st(float* p, df v) { *p = df_to_f32(v); }
 __device__ __forceinline__ df zp_f2(float2 v) { return df{v.x, v.y}; }
 __device__ __forceinline__ df zp_f2(const float* v) { return df{v[0], v[1]}; }
-
-// (A, B) pairs of one carry's segment totals: up to 16 warps x 8 lines, two words each
-constexpr int kZpAgg = 2 * 16 * 8;
 
 // Composition of chunk maps x -> A x + B: (X o Y)(x) = X(Y(x)) = (A_X A_Y) x + (A_X B_Y + B_X).
 __device__ __forceinline__ void zp_compose(df& A, df& B, df Ay, df By) {
@@ -54,48 +64,64 @@ __device__ __forceinline__ df zp_shfl(df v, int delta, bool up) {
             : df{__shfl_down_sync(0xffffffffu, v.hi, delta), __shfl_down_sync(0xffffffffu, v.lo, delta)};
 }
 
-// Carry of every chunk from the chunk maps of its line, by recursive doubling in two levels.  A warp
-// holds CW = 32 / G consecutive chunks of each of the CTA's G lines (lane = chunk-in-warp x G +
-// line), one segment per line; the warp's segments are scanned with shuffles (log2 CW levels: at
-// level o a chunk composes its map with the one o chunks nearer the start of the recurrence), the
-// segment totals are exchanged through shared memory (one barrier), and each chunk composes the
-// totals of the segments before its own.
-// dir = +1 (forward recurrence, starting at chunk 0): returns the value entering the chunk, the
-// output of chunk c - 1 (0 for chunk 0).  dir = -1 (backward recurrence, starting at the last
-// chunk): the output of chunk c + 1 (0 for the last).
-// agg: NS x G pairs of (A, B), NS = warps of the CTA.  Every thread calls it; chunks past the line
-// (c >= P) hold the identity map, which composes away.
-__device__ __forceinline__ df zp_carry(df A, df B, float2* agg, int c, int col, int G, int lgG, int dir) {
+// Terms of the carry that a thread sums itself; a mode that needs more takes the doubling.
+constexpr int kZpWindow = 8;
+
+// Carry of every chunk from the chunk maps of its line.  dir = +1 (forward recurrence): the value
+// that leaves chunk c - 1 (0 for chunk 0); dir = -1 (backward): the one that leaves chunk c + 1 (0 for
+// the last).  sA, sB: one entry per thread.  Every thread of the CTA calls it, with the same `wide`;
+// threads past the line (c >= P) hold the identity map.  `terms`: predecessors that matter to the
+// thread's mode (windowed form).  Contains one barrier.
+//
+// Doubling (wide): a warp holds CW = 32 / G consecutive chunks of each of the CTA's G lines (lane =
+// chunk-in-warp x G + line), one segment per line; the segments are scanned with shuffles (log2 CW
+// levels: at level o a chunk composes its map with the one o chunks nearer the start), the segment
+// totals are exchanged through shared memory, and each chunk composes the totals of the segments
+// before its own.
+__device__ __forceinline__ df zp_carry(df A, df B, float2* sA, float2* sB, int c, int P, int col, int G, int lgG,
+                                       int dir, bool wide, int terms) {
+  const bool fwd = dir > 0;
+  if (!wide) {
+    sA[threadIdx.x] = make_float2(A.hi, A.lo);
+    sB[threadIdx.x] = make_float2(B.hi, B.lo);
+    __syncthreads();
+    const int have = fwd ? c : P - 1 - c;
+    const int nt = min(have, terms);
+    df x = df{0.f, 0.f};
+    if (nt > 0) {
+      int t = (int)threadIdx.x - dir * (nt << lgG);  // farthest chunk that matters
+      x = zp_f2(sB[t]);
+      for (int j = 1; j < nt; j++) {
+        t += dir * G;
+        x = zp_f2(sA[t]) * x + zp_f2(sB[t]);
+      }
+    }
+    return x;
+  }
   const int lane = (int)threadIdx.x & 31;
   const int cw = 32 >> lgG;          // chunks per warp and line
   const int ci = lane >> lgG;        // chunk within the warp's segment
   const int seg = (int)threadIdx.x >> 5;
   const int nseg = ((int)blockDim.x + 31) >> 5;
-  const bool fwd = dir > 0;
   // 1. inclusive scan within the segment
   for (int o = 1; o < cw; o <<= 1) {
     const df An = zp_shfl(A, o * G, fwd), Bn = zp_shfl(B, o * G, fwd);
     if (fwd ? (ci >= o) : (ci + o < cw)) zp_compose(A, B, An, Bn);
   }
   // the inclusive map of the neighbouring chunk nearer the start (same segment unless at its edge)
-  const df An1 = zp_shfl(A, G, fwd), Bn1 = zp_shfl(B, G, fwd);
+  const df An1 = zp_shfl(A, G & 31, fwd), Bn1 = zp_shfl(B, G & 31, fwd);
   // 2. segment totals: the last chunk of a forward segment, the first of a backward one
-  float2* sA = agg;
-  float2* sB = agg + nseg * G;
   if (fwd ? (ci == cw - 1) : (ci == 0)) {
     sA[seg * G + col] = make_float2(A.hi, A.lo);
     sB[seg * G + col] = make_float2(B.hi, B.lo);
   }
   __syncthreads();
   // 3. L: the composition of the segments before this one (forward: segments 0 .. seg-1, applied
-  // in that order; backward: the last segment down to seg+1)
-  df La = df{1.f, 0.f}, Lb = df{0.f, 0.f};
+  // in that order; backward: the last segment down to seg+1); only its value at 0 is needed
+  df Lb = df{0.f, 0.f};
   for (int t = 0; t < (fwd ? seg : nseg - 1 - seg); t++) {
     const int j = fwd ? t : nseg - 1 - t;
-    df Aj = zp_f2(sA[j * G + col]), Bj = zp_f2(sB[j * G + col]);
-    zp_compose(Aj, Bj, La, Lb);  // L = Agg_j o L
-    La = Aj;
-    Lb = Bj;
+    Lb = zp_f2(sA[j * G + col]) * Lb + zp_f2(sB[j * G + col]);
   }
   // the carry: the neighbour's output, its segment map applied to L's output (at the segment's
   // edge, L's output itself)
@@ -103,104 +129,125 @@ __device__ __forceinline__ df zp_carry(df A, df B, float2* agg, int c, int col, 
   return edge ? Lb : An1 * Lb + Bn1;
 }
 
-// The multiplier of row k (table prefix, converged value, last row), as stored (pp_zmul.cuh).
+// The multipliers of a line, as stored (pp_zmul.cuh).
 struct ZpW {
-  const float2* wt;
-  int wlen, n;
-  bool plus1;  // the table holds w but the thread runs the near -1 form: convert to 1 + w
-  df winf, wlast;
-  __device__ __forceinline__ df operator()(int k) const {
-    if (k == n - 1) return wlast;
-    if (k < wlen) {
-      const df x = zp_f2(__ldg(wt + k));
-      return plus1 ? x + df{1.f, 0.f} : x;
-    }
-    return winf;
+  const float2* wt;  // prefix, wlen entries
+  int wlen;
+  bool plus1;        // the table holds w but the thread runs the near -1 form: converts to 1 + w
+  df winf, wlast;    // converged, and of the last row
+};
+
+// How a warp runs its rows.
+//  ZP_FAST: every row of every lane is past the table prefix and not the last one, so w = winf
+//           throughout.
+//  ZP_TAB:  the multipliers come from the thread's rows of sW in shared memory.  (Taken row after row
+//           from the table where they were used, and only by the lanes that needed them, they made the
+//           prefix warps of a CTA three times as slow as the others, which waited at the barriers.)
+//  ZP_WIDE: the same for a CTA whose carries reach further than the window.
+//  ZP_NEAR: the same with the near -1 form of the products (pp_zmul.cuh).
+// Inside the window the first run of a recurrence only feeds carries that enter scaled by A < 2^-7, so
+// it keeps its pairs unnormalised (12 instructions a step instead of 18; their 2^-46 is far below the
+// rounding of the second run).
+enum { ZP_FAST = 0, ZP_TAB = 1, ZP_WIDE = 2, ZP_NEAR = 3 };
+
+// Steps of the recurrences: unnormalised for the FP32 spill (as in the sweeps, pp_zsolve.cu: zr_fwd,
+// zr_bwd); for the double-float spill the value that goes on is normalised, the difference or product it
+// comes from is not (products and sums read unnormalised pairs: 15 instructions instead of 18).
+template <class S, int V, bool FIRST> __device__ __forceinline__ df zp_step_f(df d, df g, df w) {
+  if constexpr (V != ZP_NEAR && (sizeof(S) == 4 || (V <= ZP_TAB && FIRST))) return mul_u(add_u(d, -g), w);
+  else if constexpr (V == ZP_NEAR) return zw_mul<true>(d - g, w);
+  else return add_u(d, -g) * w;
+}
+template <class S, int V, bool FIRST> __device__ __forceinline__ df zp_step_b(df g, df w, df u) {
+  if constexpr (V != ZP_NEAR && (sizeof(S) == 4 || (V <= ZP_TAB && FIRST))) return add_u(g, -mul_u(w, u));
+  else if constexpr (V == ZP_NEAR) return zw_sub<true>(g, w, u);
+  else return g - mul_u(w, u);
+}
+
+struct ZpRows {
+  df winf;
+  const float2* w;  // multipliers of the thread's rows
+  template <int V> __device__ __forceinline__ df mult(int i) const {
+    if constexpr (V == ZP_FAST) return winf;
+    else return zp_f2(w[i]);
   }
 };
 
-// chunks of 16 rows keep their multipliers in registers across the four passes (measured: at 8 rows
-// the extra registers halve the resident CTAs, at 32 they spill)
-template <int M> struct ZpCacheW { static constexpr bool v = M == 16; };
-
-// The four passes over a thread's M rows, with the chunk's multipliers wv loaded once (FAST: every
-// row past the table prefix and not the last row, so w = winf throughout and wv is not read).  No
-// barrier inside: a CTA's threads may take different variants.
-// 1. forward recurrence from a zero carry: v = local g, (A, B) = the chunk's map
-template <int M, bool N1, bool FAST>
-__device__ __forceinline__ void zp_fwd(df (&v)[M], df& A, df& B, const ZpW& W, const df (&wv)[M], int k0, df scale, float& dmax) {
+// Rows past the line's end (the last chunk) have d = 0 and w = -1, which pass g and u on unchanged.
+// scaled right-hand sides d_k in place of the raw values, and the value that leaves the chunk
+template <class S, int M, int V>
+__device__ __forceinline__ void zp_fwd1(df (&v)[M], df& B, const ZpRows& R, df scale, float& dmax) {
 #pragma unroll
   for (int i = 0; i < M; i++) {
-    const int k = k0 + i;
-    if (FAST || k < W.n) {
-      const df d = v[i] * scale;
-      track(dmax, d.hi);
-      const df w = FAST ? W.winf : (ZpCacheW<M>::v ? wv[i] : W(k));
-      B = zw_mul<N1>(d - B, w);
-      A = zw_neg_mul<N1>(A, w);
-      v[i] = B;
-    }
+    v[i] = (sizeof(S) == 4) ? mul_u(v[i], scale) : v[i] * scale;
+    track(dmax, v[i].hi);
+    B = zp_step_f<S, V, true>(v[i], B, R.mult<V>(i));
   }
 }
-// 2. g_k = local g_k + (a_k0 ... a_k) g_in
-template <int M, bool N1, bool FAST>
-__device__ __forceinline__ void zp_fwd_fix(df (&v)[M], df gin, const ZpW& W, const df (&wv)[M], int k0) {
-  df Pk = df{1.f, 0.f};
+// g_k from the true carry, in place of d_k; rounded for the FP32 spill as the sweeps round it between
+// their two passes, so that both give a plan the same results but for rare last-place flips
+template <class S, int M, int V>
+__device__ __forceinline__ void zp_fwd2(df (&v)[M], df& g, const ZpRows& R) {
 #pragma unroll
   for (int i = 0; i < M; i++) {
-    const int k = k0 + i;
-    if (FAST || k < W.n) {
-      Pk = zw_neg_mul<N1>(Pk, FAST ? W.winf : (ZpCacheW<M>::v ? wv[i] : W(k)));
-      v[i] = v[i] + Pk * gin;
-    }
+    g = zp_step_f<S, V, false>(v[i], g, R.mult<V>(i));
+    v[i] = (sizeof(S) == 4) ? df{df_to_f32(g), 0.0f} : g;
   }
 }
-// 3. back substitution u_k = g_k - w_k u_{k+1} from a zero carry above the chunk
-template <int M, bool N1, bool FAST>
-__device__ __forceinline__ void zp_bwd(df (&v)[M], df& A, df& B, const ZpW& W, const df (&wv)[M], int k0) {
+// back substitution u_k = g_k - w_k u_{k+1}: the value that leaves the chunk
+template <class S, int M, int V>
+__device__ __forceinline__ void zp_bwd1(const df (&v)[M], df& u, const ZpRows& R) {
 #pragma unroll
-  for (int i = M - 1; i >= 0; i--) {
-    const int k = k0 + i;
-    if (FAST || k < W.n) {
-      const df w = FAST ? W.winf : (ZpCacheW<M>::v ? wv[i] : W(k));
-      B = zw_sub<N1>(v[i], w, B);
-      A = zw_neg_mul<N1>(A, w);
-      v[i] = B;
-    }
-  }
+  for (int i = M - 1; i >= 0; i--) u = zp_step_b<S, V, true>(v[i], R.mult<V>(i), u);
 }
-// 4. u_k = local u_k + (a_k ... a_end) u_in
-template <int M, bool N1, bool FAST>
-__device__ __forceinline__ void zp_bwd_fix(df (&v)[M], df uin, const ZpW& W, const df (&wv)[M], int k0) {
-  df Qk = df{1.f, 0.f};
+// ... and from the true carry, keeping the values
+template <class S, int M, int V>
+__device__ __forceinline__ void zp_bwd2(df (&v)[M], df u, const ZpRows& R) {
 #pragma unroll
   for (int i = M - 1; i >= 0; i--) {
-    const int k = k0 + i;
-    if (FAST || k < W.n) {
-      Qk = zw_neg_mul<N1>(Qk, FAST ? W.winf : (ZpCacheW<M>::v ? wv[i] : W(k)));
-      v[i] = v[i] + Qk * uin;
-    }
+    u = zp_step_b<S, V, false>(v[i], R.mult<V>(i), u);
+    v[i] = u;
   }
 }
 
-#define ZP_DISPATCH(fn, ...)                                       \
-  do {                                                             \
-    if (fast) {                                                    \
-      if (n1) fn<M, true, true>(__VA_ARGS__);                      \
-      else fn<M, false, true>(__VA_ARGS__);                        \
-    } else {                                                       \
-      if (n1) fn<M, true, false>(__VA_ARGS__);                     \
-      else fn<M, false, false>(__VA_ARGS__);                       \
-    }                                                              \
+#define ZP_DISPATCH(fn, ...)                               \
+  do {                                                     \
+    if (var == ZP_FAST) fn<S, M, ZP_FAST>(__VA_ARGS__);    \
+    else if (var == ZP_TAB) fn<S, M, ZP_TAB>(__VA_ARGS__); \
+    else if (var == ZP_WIDE) fn<S, M, ZP_WIDE>(__VA_ARGS__); \
+    else fn<S, M, ZP_NEAR>(__VA_ARGS__);                   \
   } while (0)
 
-template <class S, int M>
-__global__ void __launch_bounds__(512) k_zpart(const ZArgs a, int G, int lgG, int P) {
-  __shared__ float2 zp_sm[2 * kZpAgg];  // segment totals of the forward and the backward carries
+// x^M for the chunk's map, M a power of two
+template <int M> __device__ __forceinline__ df zp_pow(df x) {
+#pragma unroll
+  for (int m = 1; m < M; m <<= 1) x = x * x;
+  return x;
+}
+
+// CTAs of up to 1024 threads at 64 registers (8 or 16 rows a thread), 512 at 128 (32 rows)
+template <int M> struct ZpThreads { static constexpr int v = M <= 16 ? 1024 : 512; };
+
+template <class S, int M, bool PER>
+__global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G, int lgG, int P) {
+  // per-thread chunk maps (A, B) of the forward and the backward carries; periodic z: partial sums
+  // of y_0, and c per line
+  extern __shared__ float2 zp_sm[];
+  float dmax = 0.0f, umax = 0.0f;
+  if ((int)blockIdx.x < a.nsing) {
+    zsing_block<S>(a, (int)blockIdx.x, zp_sm, dmax, umax);
+    range_report(a.rstat, a.dmin, a.umax, gridDim.x, dmax, umax);
+    return;
+  }
+  const int T = (int)blockDim.x;
+  float2 *fA = zp_sm, *fB = zp_sm + T, *bA = zp_sm + 2 * T, *bB = zp_sm + 3 * T;
+  float2* sW = zp_sm + 4 * T + (int)threadIdx.x * (M + 1);  // M entries a thread (odd stride: no bank conflicts)
+  float2* sQ = zp_sm + (5 + M) * T;  // T entries
+  float2* sC = sQ + T;               // G entries
   const int tid = (int)threadIdx.x;
   const int col = tid & (G - 1);
   const int c = tid >> lgG;
-  const long long s = (long long)blockIdx.x * G + col;
+  const long long s = (long long)((int)blockIdx.x - a.nsing) * G + col;
   const int n = a.nz;
   const long long PL = a.plane;
 
@@ -218,100 +265,191 @@ __global__ void __launch_bounds__(512) k_zpart(const ZArgs a, int G, int lgG, in
       live = !(m->flags & ZF_SINGULAR);
     }
   }
+  const int k0 = c * M;
+  const int nr = max(0, min(M, n - k0));  // rows of the chunk (below M only at the line's end)
+  S* base = reinterpret_cast<S*>(a.data) + s + (long long)k0 * PL;
+  df v[M];
+  if (live && nr == M) {
+#pragma unroll
+    for (int i = 0; i < M; i++) v[i] = zp_ld(base + (long long)i * PL);
+  } else {
+#pragma unroll
+    for (int i = 0; i < M; i++) v[i] = (live && i < nr) ? zp_ld(base + (long long)i * PL) : df{0.f, 0.f};
+  }
   ZpW W;
   W.wt = a.wtab;
   W.wlen = 0;
-  W.n = n;
   W.winf = df{0.f, 0.f};
   W.wlast = df{0.f, 0.f};
   bool mine = false;
+  int qlen = 0;
   if (live) {
-    W.winf = zp_f2(m->winf);
-    W.wlast = zp_f2(m->wlast);
-    W.wlen = m->wlen;
-    W.wt = a.wtab + m->woff;
+    const int4 off = __ldg(reinterpret_cast<const int4*>(m));          // woff, wlen, qoff, qlen
+    const float4 ww = __ldg(reinterpret_cast<const float4*>(m) + 1);   // winf, wlast
+    W.winf = df{ww.x, ww.y};
+    W.wlast = df{ww.z, ww.w};
+    W.wlen = off.y;
+    W.wt = a.wtab + off.x;
     mine = (m->flags & ZF_NEAR1) != 0;
+    if (PER) qlen = off.w;
   }
-  // a warp runs the near -1 form when any of its modes needs it (the others convert their w)
+  // a warp runs the near -1 form when any of its modes needs it (the others convert their w); every
+  // warp holds all G lines, so all warps of the CTA agree
   const bool n1 = __any_sync(0xffffffffu, mine);
   W.plus1 = n1 && !mine;
   if (W.plus1) {
     W.winf = W.winf + df{1.f, 0.f};
     W.wlast = W.wlast + df{1.f, 0.f};
   }
-  const int k0 = c * M;
-  // a chunk past the multiplier prefix that does not hold the last row uses winf throughout
-  const bool fast = k0 >= W.wlen && k0 + M < n;
   const df scale = df{a.scale[0], a.scale[1]};
-  S* base = reinterpret_cast<S*>(a.data) + s;
-  float dmax = 0.0f, umax = 0.0f;
-  // the chunk's multipliers, loaded once for the four passes (chunks in the table prefix)
-  df wv[M];
-#pragma unroll
-  for (int i = 0; i < M; i++) wv[i] = (ZpCacheW<M>::v && !fast && k0 + i < n) ? W(k0 + i) : W.winf;
 
-  df v[M];
-#pragma unroll
-  for (int i = 0; i < M; i++) {
-    const int k = k0 + i;
-    v[i] = (live && k < n) ? zp_ld(base + (long long)k * PL) : df{0.f, 0.f};
-  }
-
-  // forward recurrence: local pass, carries by recursive doubling, fix-up
-  df A = df{1.f, 0.f}, B = df{0.f, 0.f};
-  ZP_DISPATCH(zp_fwd, v, A, B, W, wv, k0, scale, dmax);
-  const df gin = zp_carry(A, B, zp_sm, c, col, G, lgG, +1);
-  if (inb && c > 0) ZP_DISPATCH(zp_fwd_fix, v, gin, W, wv, k0);
-
-  // back substitution: the same three steps from the top of each chunk
-  A = df{1.f, 0.f};
-  B = df{0.f, 0.f};
-  ZP_DISPATCH(zp_bwd, v, A, B, W, wv, k0);
-  const df uin = zp_carry(A, B, zp_sm + kZpAgg, c, col, G, lgG, -1);
-  if (c + 1 < P) ZP_DISPATCH(zp_bwd_fix, v, uin, W, wv, k0);
-  if (live) {
+  // A of a converged chunk and how many chunks back it reaches
+  df A = zp_pow<M>(n1 ? df{1.f, 0.f} - W.winf : -W.winf);
+  const int terms = A.hi < 0x1p-56f ? 1 : (int)__fdividef(-56.0f, __log2f(fminf(A.hi, 0.999f))) + 1;
+  const bool wide = __any_sync(0xffffffffu, live && terms > kZpWindow);
+  const bool lanes_fast = __all_sync(0xffffffffu, k0 >= W.wlen && k0 + M < n);
+  const int var = n1 ? ZP_NEAR : (wide ? ZP_WIDE : (lanes_fast ? ZP_FAST : ZP_TAB));
+  ZpRows R;
+  R.winf = W.winf;
+  R.w = sW;
+  if (var != ZP_FAST) {
+    // the chunk's multipliers, read back by this thread only: asynchronous copies of the table's part
 #pragma unroll
     for (int i = 0; i < M; i++) {
       const int k = k0 + i;
-      if (k < n) {
-        track(umax, v[i].hi);
-        zp_st(base + (long long)k * PL, v[i]);
+      if (k < W.wlen && k < n - 1) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(sW + i)),
+                     "l"(__cvta_generic_to_global(W.wt + k)) : "memory");
+      } else {
+        const df w = k < n - 1 ? W.winf : (k == n - 1 ? W.wlast : df{n1 ? 0.f : -1.f, 0.f});
+        sW[i] = make_float2(w.hi, w.lo);
       }
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if (W.plus1)
+      for (int i = 0; i < M && k0 + i < min(W.wlen, n - 1); i++) {
+        const df w = zp_f2(sW[i]) + df{1.f, 0.f};
+        sW[i] = make_float2(w.hi, w.lo);
+      }
+    // A of a chunk in the prefix (nothing passes through the first chunk, or through the last)
+    if (k0 < W.wlen && c > 0 && c < P - 1) {
+      A = df{1.f, 0.f};
+#pragma unroll
+      for (int i = 0; i < M; i++) A = n1 ? zw_neg_mul<true>(A, zp_f2(sW[i])) : zw_neg_mul<false>(A, zp_f2(sW[i]));
+    }
+  }
+
+  // forward recurrence
+  df B = df{0.f, 0.f};
+  ZP_DISPATCH(zp_fwd1, v, B, R, scale, dmax);
+  if (PER) {
+    df y0 = df{0.f, 0.f};
+    if (k0 < qlen) {
+#pragma unroll
+      for (int i = 0; i < M; i++)
+        if (k0 + i < qlen) y0 = y0 + zp_f2(__ldg(a.qtab + m->qoff + k0 + i)) * v[i];
+    }
+    sQ[tid] = make_float2(y0.hi, y0.lo);
+  }
+  df x = zp_carry(A, B, fA, fB, c, P, col, G, lgG, +1, wide, terms);
+  ZP_DISPATCH(zp_fwd2, v, x, R);
+
+  // back substitution; periodic z starts it from c = (y_0 + y_{n-1} / gamma) / (1 + z_0 + z_{n-1} / gamma)
+  df top = df{0.f, 0.f};
+  if (PER && live && c == P - 1) {
+    df y0 = df{0.f, 0.f};
+    for (int j = 0; j * M < qlen; j++) y0 = y0 + zp_f2(sQ[(j << lgG) + col]);
+    top = (y0 + x * zp_f2(m->igam)) * zp_f2(m->dsm);  // x == y_{n-1}
+    sC[col] = make_float2(top.hi, top.lo);
+  }
+  if (nr < M) {
+#pragma unroll
+    for (int i = 0; i < M; i++)
+      if (i >= nr) v[i] = df{0.f, 0.f};
+  }
+  B = top;
+  ZP_DISPATCH(zp_bwd1, v, B, R);
+  x = zp_carry(A, B, bA, bB, c, P, col, G, lgG, -1, wide, terms);
+  if (c == P - 1) x = top;
+  ZP_DISPATCH(zp_bwd2, v, x, R);
+  if (live) {
+    if (PER && k0 < qlen) {
+      const df cg = zp_f2(sC[col]) * zp_f2(m->gam);
+#pragma unroll
+      for (int i = 0; i < M; i++)
+        if (k0 + i < qlen) v[i] = v[i] - cg * zp_f2(__ldg(a.qtab + m->qoff + k0 + i));
+    }
+    if (nr == M) {
+#pragma unroll
+      for (int i = 0; i < M; i++) {
+        track(umax, v[i].hi);
+        zp_st(base + (long long)i * PL, v[i]);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < M; i++)
+        if (i < nr) {
+          track(umax, v[i].hi);
+          zp_st(base + (long long)i * PL, v[i]);
+        }
     }
   }
   range_report(a.rstat, a.dmin, a.umax, gridDim.x, dmax, umax);
 }
 #undef ZP_DISPATCH
 
-// Chunk count P = ceil(nz / M) and slots per CTA G (a power of two, G P <= 512, G <= 8; the CTA
-// is G P threads rounded up to whole warps); returns false when a line needs more than 512 chunks.
-bool zpart_shape(int nz, int M, int* G, int* lgG, int* P) {
+// Chunk count P = ceil(nz / M) and slots per CTA G (a power of two up to 16; the CTA is G P threads
+// rounded up to whole warps); false when a line needs more than 512 chunks.  CTAs of up to 512
+// threads, two or more of which share an SM (one loads while another computes), as long as a row's
+// segment keeps 64 bytes; larger ones down to whole 32-byte sectors where the line is longer.
+bool zpart_shape(int nz, int M, int elem, int* G, int* lgG, int* P) {
   const int p = (nz + M - 1) / M;
   if (p > 512) return false;
-  int g = 8, lg = 3;
-  while (g > 1 && g * p > 512) { g >>= 1; lg--; }
+  const int tmax = M <= 16 ? 1024 : 512;
+  int g = 16, lg = 4;
+  while (g * elem > 64 && g * p > 512) { g >>= 1; lg--; }
+  while (g > 1 && g * p > tmax) { g >>= 1; lg--; }
   *G = g; *lgG = lg; *P = p;
   return true;
 }
 
-template <class S, int M>
+template <class S, int M, bool PER>
 static cudaError_t launch_zpart_t(const ZArgs& a, cudaStream_t st) {
   int G, lgG, P;
-  if (!zpart_shape(a.nz, M, &G, &lgG, &P)) return cudaErrorInvalidConfiguration;
-  const long long grid = (a.nreal + G - 1) / G;
+  if (!zpart_shape(a.nz, M, (int)sizeof(S), &G, &lgG, &P)) return cudaErrorInvalidConfiguration;
+  const long long grid = (a.nreal + G - 1) / G + a.nsing;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   const int threads = (G * P + 31) / 32 * 32;  // whole warps (the scans and the range report shuffle)
-  k_zpart<S, M><<<(unsigned)grid, threads, 0, st>>>(a, G, lgG, P);
+  const size_t sm = std::max(sizeof(float2) * ((5 + M + (PER ? 1 : 0)) * (size_t)threads + (PER ? G : 0)), kZsingSmem);
+  // dynamic shared memory above 48 KB must be opted into, per device (one bit per device ordinal below
+  // 64; higher ordinals set the attribute on every launch)
+  static std::atomic<unsigned long long> attr_done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = (dev >= 0 && dev < 64) ? (1ull << dev) : 0ull;
+  if (!bit || !(attr_done.load(std::memory_order_acquire) & bit)) {
+    e = cudaFuncSetAttribute(k_zpart<S, M, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
+    if (e != cudaSuccess) return e;
+    attr_done.fetch_or(bit, std::memory_order_release);
+  }
+  k_zpart<S, M, PER><<<(unsigned)grid, threads, sm, st>>>(a, G, lgG, P);
   return cudaGetLastError();
 }
 
-cudaError_t launch_zpart_impl(const ZArgs& a, bool df_spill, int M, cudaStream_t st) {
+template <class S, bool PER>
+static cudaError_t launch_zpart_m(const ZArgs& a, int M, cudaStream_t st) {
   switch (M) {
-    case 8: return df_spill ? launch_zpart_t<float2, 8>(a, st) : launch_zpart_t<float, 8>(a, st);
-    case 16: return df_spill ? launch_zpart_t<float2, 16>(a, st) : launch_zpart_t<float, 16>(a, st);
-    case 32: return df_spill ? launch_zpart_t<float2, 32>(a, st) : launch_zpart_t<float, 32>(a, st);
+    case 8: return launch_zpart_t<S, 8, PER>(a, st);
+    case 16: return launch_zpart_t<S, 16, PER>(a, st);
+    case 32: return launch_zpart_t<S, 32, PER>(a, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_zpart_impl(const ZArgs& a, bool df_spill, bool zper, int M, cudaStream_t st) {
+  if (df_spill) return zper ? launch_zpart_m<float2, true>(a, M, st) : launch_zpart_m<float2, false>(a, M, st);
+  return zper ? launch_zpart_m<float, true>(a, M, st) : launch_zpart_m<float, false>(a, M, st);
 }
 
 }  // namespace pp

@@ -23,14 +23,15 @@
 //     v_k = g_k - w_k v_{k+1},  v_{n-1} = g_{n-1} - c w_{n-1},
 // and x_k = v_k - c gamma q_k: the cyclic solve takes the two Thomas sweeps plus the q prefix.
 //
-// The singular mode of a problem without Dirichlet faces (Sec. "Well-posedness") removes the
-// source mean, pins u_0 = 0, solves rows 1..n-1, and shifts the result to zero mean.
+// The singular mode of a problem without Dirichlet faces (Sec. "Well-posedness") is solved by CTAs of
+// its own, one for each of its real slots, at the front of the grid (pp_zsing.cuh).
 //
 // All arithmetic is double-float (pp_arith.cuh), whatever the storage type of the spill.
 //
 // Range report: see pp_range.cuh (largest scaled input and output per launch).
 #include "pp_range.cuh"
 #include "pp_zmul.cuh"
+#include "pp_zsing.cuh"
 
 namespace pp {
 
@@ -78,51 +79,6 @@ __device__ __forceinline__ void zload_batch(S* v, const S* base, long long P, in
   const int klast = k0 + step * (ZU - 1);
   if (k0 >= 0 && k0 < n && klast >= 0 && klast < n) zload_full<ZU>(v, base + (long long)k0 * P, P32, step);
   else zload<ZU>(v, base, P, k0, step, n);
-}
-
-// The singular mode: remove the source mean, pin u_0 = 0, solve rows 1..n-1, shift to zero mean.
-template <class S>
-__device__ __noinline__ void z_singular(S* base, long long P, int n, df scale, const float2* wt, float& dmax,
-                                        float& umax) {
-  // The pinned system is consistent only for a zero-mean right-hand side; a remainder c of the mean
-  // would add a profile growing like c k^2 / 2.  One double-float pass leaves the rounding of a sum
-  // of n values of the source's own mean magnitude (relative 2^-48 per term), so a second pass takes
-  // the mean of the residuals, which are of the size of the fluctuations.
-  const df rn = df_rcp(df{(float)n, 0.f});
-  df sum = df{0.f, 0.f};
-  for (int k = 0; k < n; k++) sum = sum + zcvt(base[k * P]);
-  df mean = sum * rn;
-  df rsum = df{0.f, 0.f};
-  for (int k = 0; k < n; k++) rsum = rsum + (zcvt(base[k * P]) - mean);
-  mean = mean + rsum * rn;
-  // rows 1..n-1 of the pinned system; multipliers of the sub-system in the table
-  df g = df{0.f, 0.f};
-  for (int k = 1; k < n; k++) {
-    df d = (zcvt(base[k * P]) - mean) * scale;
-    track(dmax, d.hi);
-    g = zw_mul<true>(d - g, f2df(__ldg(wt + (k - 1))));  // the pinned table is stored as 1 + w
-    zput(base + k * P, g);
-  }
-  df u = df{0.f, 0.f};
-  df usum = df{0.f, 0.f};
-  for (int k = n - 1; k >= 1; k--) {
-    df gk = zcvt(base[k * P]);
-    u = (k == n - 1) ? gk : zw_sub<true>(gk, f2df(__ldg(wt + (k - 1))), u);
-    usum = usum + u;
-    zput(base + k * P, u);
-  }
-  df umean = usum * rn;
-  // the same second pass for the solution's mean (u_0 = 0 is pinned)
-  df ursum = -umean;
-  for (int k = 1; k < n; k++) ursum = ursum + (zcvt(base[k * P]) - umean);
-  umean = umean + ursum * rn;
-  zput(base, -umean);
-  track(umax, umean.hi);
-  for (int k = 1; k < n; k++) {
-    const df v = zcvt(base[k * P]) - umean;
-    track(umax, v.hi);
-    zput(base + k * P, v);
-  }
 }
 
 // Steps of the Thomas recurrences, g_k = (d_k - g_{k-1}) w_k and u_k = g_k - w_k u_{k+1}.  The
@@ -303,7 +259,7 @@ __device__ __noinline__ void z_sweeps_near1(const ZArgs& a, const ZMode& m, S* b
 
 template <class S, int MODE>
 __device__ __forceinline__ void z_line(const ZArgs& a, float& dmax, float& umax) {
-  long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long s = (long long)((int)blockIdx.x - a.nsing) * blockDim.x + threadIdx.x;
   if (s >= a.nreal) return;
   // slot s of the (padded) spectral plane -> row, column; padding columns carry no mode
   const unsigned row = a.fd_row.div((unsigned)s);
@@ -317,11 +273,7 @@ __device__ __forceinline__ void z_line(const ZArgs& a, float& dmax, float& umax)
   const df scale = df{a.scale[0], a.scale[1]};
   const float2* wt = a.wtab + m.woff;
   const int flags = m.flags;
-  if (a.only_singular && !(flags & ZF_SINGULAR)) return;
-  if (flags & ZF_SINGULAR) {
-    z_singular<S>(base, P, n, scale, wt, dmax, umax);
-    return;
-  }
+  if (flags & ZF_SINGULAR) return;
   // a warp runs the near -1 form when any of its modes needs it (the others convert their w): no
   // warp runs both forms one after the other
   const bool mine = (flags & ZF_NEAR1) != 0;
@@ -511,7 +463,7 @@ __device__ __noinline__ void z_sweeps_ck_near1(const ZArgs& a, const ZMode& m, f
 template <int MODE>
 __device__ __forceinline__ void z_line_ck(const ZArgs& a, float& dmax, float& umax) {
   using S = float2;
-  long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long s = (long long)((int)blockIdx.x - a.nsing) * blockDim.x + threadIdx.x;
   if (s >= a.nreal) return;
   const unsigned row = a.fd_row.div((unsigned)s);
   const int col = (int)(s - (long long)row * a.row_reals);
@@ -524,11 +476,7 @@ __device__ __forceinline__ void z_line_ck(const ZArgs& a, float& dmax, float& um
   const int n = a.nz;
   const df scale = df{a.scale[0], a.scale[1]};
   const float2* wt = a.wtab + m.woff;
-  if (a.only_singular && !(m.flags & ZF_SINGULAR)) return;
-  if (m.flags & ZF_SINGULAR) {
-    z_singular<S>(base, P, n, scale, wt, dmax, umax);
-    return;
-  }
+  if (m.flags & ZF_SINGULAR) return;
   const bool mine = (m.flags & ZF_NEAR1) != 0;
   if (__any_sync(__activemask(), mine))
     z_sweeps_ck_near1<MODE>(a, m, base, ck, P, CP, n, scale, wt, !mine, dmax, umax);
@@ -542,14 +490,18 @@ template <int MODE> struct ZCkMinBlocks { static constexpr int v = (MODE == 1) ?
 template <int MODE>
 __global__ void __launch_bounds__(256, (ZCkMinBlocks<MODE>::v)) k_zsolve_ck(const ZArgs a) {
   float dmax = 0.0f, umax = 0.0f;
-  z_line_ck<MODE>(a, dmax, umax);
+  __shared__ float2 sm[kZsingSmem / sizeof(float2)];
+  if ((int)blockIdx.x < a.nsing) zsing_block<float2>(a, (int)blockIdx.x, sm, dmax, umax);
+  else z_line_ck<MODE>(a, dmax, umax);
   range_report(a.rstat, a.dmin, a.umax, gridDim.x, dmax, umax);
 }
 
 template <class S, int MODE>
 __global__ void __launch_bounds__(256, (ZMinBlocks<S, MODE>::v)) k_zsolve(const ZArgs a) {
   float dmax = 0.0f, umax = 0.0f;
-  z_line<S, MODE>(a, dmax, umax);
+  __shared__ float2 sm[kZsingSmem / sizeof(float2)];
+  if ((int)blockIdx.x < a.nsing) zsing_block<S>(a, (int)blockIdx.x, sm, dmax, umax);
+  else z_line<S, MODE>(a, dmax, umax);
   range_report(a.rstat, a.dmin, a.umax, gridDim.x, dmax, umax);
 }
 
@@ -562,9 +514,8 @@ static cudaError_t launch_z(const ZArgs& a, int mode, unsigned grid, int threads
 }
 
 cudaError_t launch_zsolve_impl(const ZArgs& a, bool df_spill, bool zper, cudaStream_t st) {
-  // the singular mode alone: it is mode (0, 0), real slot 0 (and 1 for a complex mode)
-  const int threads = a.only_singular ? 32 : 256;
-  const long long grid = a.only_singular ? 1 : (a.nreal + threads - 1) / threads;
+  const int threads = 256;
+  const long long grid = (a.nreal + threads - 1) / threads + a.nsing;
   // periodic z is self-adjoint in this factorisation; the transposed sweep is for Thomas only
   const int mode = zper ? 1 : (a.transpose ? 2 : 0);
   if (df_spill) {
