@@ -69,7 +69,9 @@ typedef enum {
 
 /* Optional plan settings; pass NULL for the defaults. */
 typedef struct pp_plan_options {
-  int threads_x;   /* CTA size of the x-line kernels (0 = automatic) */
+  int threads_x;   /* CTA size of the x-line kernels (0 = automatic; FP64-class plans then take kernels of one
+                      fixed shape where x or y has 128 to 2048 = 2^a cells, or 64 to 1024 = 2^a complex
+                      ones, and the autotuner leaves those as they are) */
   int threads_y;   /* CTA size of the y-line kernels (0 = automatic) */
   int lines_x;     /* lines per CTA, x kernels (0 = automatic) */
   int cols_y;      /* columns per CTA, y kernels (0 = automatic) */

@@ -150,15 +150,16 @@ static __device__ __noinline__ df df_from_double_slow(double d) {
   r.hi = __uint_as_float(sign | ((unsigned)ef << 23) | mh);
   if (ef >= 24) {
     unsigned base = sign | ((unsigned)(ef - 23) << 23);
-    r.lo = __fsub_rn(__uint_as_float(base | ((l32 & 0x1fffffffu) >> 6)), __uint_as_float(base));
+    r.lo = __fsub_rn(__uint_as_float(base + (((l32 & 0x1fffffffu) + 32u) >> 6)), __uint_as_float(base));
   } else {
     r.lo = 0.0f;
   }
   return r;
 }
 
-// Split an FP64 value into hi + lo (hi = truncated 24-bit significand, lo = the next 23 bits),
-// using integer operations only.  |d| < 2^-103 keeps only hi; |d| < 2^-126 becomes the nearest
+// Split an FP64 value into hi + lo (hi = truncated 24-bit significand, lo = the rest rounded to 23 bits; a
+// carry out of them reaches the exponent and gives hi's last place, as it should), using integer
+// operations only.  |d| < 2^-103 keeps only hi; |d| < 2^-126 becomes the nearest
 // FP32 subnormal (zero below 2^-150).
 __device__ __forceinline__ df df_from_double(double d) {
   const unsigned h32 = (unsigned)__double2hiint(d), l32 = (unsigned)__double2loint(d);
@@ -169,7 +170,7 @@ __device__ __forceinline__ df df_from_double(double d) {
   r.hi = __uint_as_float(sign | __funnelshift_l(l32, t, 3));
   // lo: the 23 bits below hi's last place, as (2^(e_f-23) (1 + m/2^23)) - 2^(e_f-23)
   const unsigned base = sign | ((t - (23u << 20)) >> 20 << 23);
-  r.lo = __fsub_rn(__uint_as_float(base | ((l32 & 0x1fffffffu) >> 6)), __uint_as_float(base));
+  r.lo = __fsub_rn(__uint_as_float(base + (((l32 & 0x1fffffffu) + 32u) >> 6)), __uint_as_float(base));
   return r;
 }
 

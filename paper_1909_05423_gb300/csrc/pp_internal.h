@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "pp_fft.cuh"
+#include "pp_hx.cuh"
 #include "pittpack_gb.h"
 
 namespace pp {
@@ -56,7 +57,14 @@ struct LineArgs {
   FastDiv fd_parts;   // 1 or 2
   FastDiv fd_nblk;    // column blocks per plane
   FastDiv fd_gpc;     // y: groups of vector-width adjacent lines per CTA
+  // block-scaled kernels (pp_hlines.cuh): stage and pre/post twiddles, scale bounds, direction
+  const void* htab;
+  const void* haux;
+  HScale hs;
+  int hdir;
+  int ahead;          // tiles between the one a CTA works on and the one it prefetches into L2
 };
+constexpr int kHAhead = 152;  // LineArgs::ahead: one tile per SM (pp_hlines.cuh)
 constexpr int kMaxLpc = 512;  // lines per CTA (bounds the per-line bases in shared memory)
 constexpr int kHostChunks = 8;  // plane chunks of a host-buffer solve (copies overlap transforms)
 
@@ -64,6 +72,8 @@ constexpr int kHostChunks = 8;  // plane chunks of a host-buffer solve (copies o
 // 24..768.  Their stage twiddles are stored per stage in butterfly order (fft_lines_ct); other
 // lengths keep w_M^j, j < M.
 constexpr int kCtMin = 8, kCtMax = 1024;
+// lengths with block-scaled kernels (FP64-class plans)
+inline bool hx_length(int M) { return M >= 64 && M <= 1024 && (M & (M - 1)) == 0; }
 inline bool ct_length(int M) {
   const bool p2 = M >= kCtMin && M <= kCtMax && (M & (M - 1)) == 0;
   const int t = M / 3;
@@ -169,6 +179,9 @@ struct pp_plan {
   // launch shapes
   int threads_x[2], lpc_x[2], ldm_x;  // [0] forward, [1] inverse kernels
   int threads_y[2], lpc_y[2], ldm_y;
+  // block-scaled line kernels (pp_hlines.cuh): which stages take them ([0] forward, [1] inverse), tables
+  bool hx_x[2], hx_y[2], hx_z;
+  void* d_h_x; void* d_h_y; void* d_h_z;
   // mixed-precision refinement scratch
   void* d_resid;       // residual / correction (FP64 I/O size)
   void* d_mean;        // kMeanParts partial sums + 1 mean (float2 each), singular refinement
