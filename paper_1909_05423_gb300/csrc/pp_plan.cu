@@ -1208,12 +1208,14 @@ void evict_plan(const pp_plan* p) {
 // Launch settings of a plan that a batched graph may swap: launch shapes and the z algorithm.
 struct PlanSettings {
   int threads_x[2], lpc_x[2], ldm_x, threads_y[2], lpc_y[2], ldm_y, threads_z, lpc_z, ldm_z, zsplit, zmethod;
+  bool hx_x[2], hx_y[2];
 };
 static PlanSettings get_settings(const pp_plan* p) {
   PlanSettings s;
   for (int d = 0; d < 2; d++) {
     s.threads_x[d] = p->threads_x[d]; s.lpc_x[d] = p->lpc_x[d];
     s.threads_y[d] = p->threads_y[d]; s.lpc_y[d] = p->lpc_y[d];
+    s.hx_x[d] = p->hx_x[d]; s.hx_y[d] = p->hx_y[d];
   }
   s.ldm_x = p->ldm_x; s.ldm_y = p->ldm_y;
   s.threads_z = p->threads_z; s.lpc_z = p->lpc_z; s.ldm_z = p->ldm_z;
@@ -1225,6 +1227,7 @@ static void set_settings(pp_plan* p, const PlanSettings& s) {
   for (int d = 0; d < 2; d++) {
     p->threads_x[d] = s.threads_x[d]; p->lpc_x[d] = s.lpc_x[d];
     p->threads_y[d] = s.threads_y[d]; p->lpc_y[d] = s.lpc_y[d];
+    p->hx_x[d] = s.hx_x[d]; p->hx_y[d] = s.hx_y[d];
   }
   p->ldm_x = s.ldm_x; p->ldm_y = s.ldm_y;
   p->threads_z = s.threads_z; p->lpc_z = s.lpc_z; p->ldm_z = s.ldm_z;
@@ -1232,25 +1235,43 @@ static void set_settings(pp_plan* p, const PlanSettings& s) {
   p->zmethod = s.zmethod;
 }
 
-// Puts the autotuned members of a batch on the library's shared-GPU settings -- the default launch
-// shapes and, where the autotuner chose the z algorithm, the default one of its size (the z transform
-// buys a lone plan latency with extra work) -- for the scope of one capture, and restores their own settings afterwards (a captured graph keeps the
-// launch parameters it was captured with).
+// Puts the members of a batch on the library's shared-GPU settings for the scope of one capture, and
+// restores their own afterwards (a captured graph keeps the launch parameters it was captured with).
+//  * Every member: lines of fewer than 256 complex points take the double-float kernels.  The
+//    block-scaled ones hold twice the registers; alone on the GPU they are faster at those lengths (256^3:
+//    0.55 against 0.61 ms), beside 31 other branches their fewer resident warps are not (64 uneven grids:
+//    3.00 against 2.83 ms).
+//  * Autotuned members, if `tuned` is set: the default launch shapes and, where the autotuner chose the z
+//    algorithm, the default one of its size (the z transform buys a lone plan latency with extra work).
 struct SettingsSwap {
   std::vector<std::pair<pp_plan*, PlanSettings>> saved;
-  void apply(pp_plan* const* plans, int n) {
+  void apply(pp_plan* const* plans, int n, bool tuned) {
     for (int i = 0; i < n; i++) {
       pp_plan* p = plans[i];
-      if (!p->tuned) continue;
       bool seen = false;
       for (const auto& s : saved) seen |= (s.first == p);
       if (seen) continue;
-      saved.emplace_back(p, get_settings(p));
-      choose_shapes(p, nullptr);
-      if (p->z_tuned) {
-        p->zsplit = z_rows_default(p);
-        p->zmethod = ZM_SM;
+      const PlanSettings own = get_settings(p);
+      saved.emplace_back(p, own);
+      for (int d = 0; d < 2; d++) {
+        p->hx_x[d] = own.hx_x[d] && p->fx.M >= 256;
+        p->hx_y[d] = own.hx_y[d] && p->fy.M >= 256;
       }
+      choose_shapes(p, nullptr);
+      if (tuned && p->tuned) {
+        if (p->z_tuned) {
+          p->zsplit = z_rows_default(p);
+          p->zmethod = ZM_SM;
+        }
+        continue;
+      }
+      // the other stages keep the plan's shapes
+      for (int d = 0; d < 2; d++) {
+        if (p->hx_x[d] == own.hx_x[d]) { p->threads_x[d] = own.threads_x[d]; p->lpc_x[d] = own.lpc_x[d]; }
+        if (p->hx_y[d] == own.hx_y[d]) { p->threads_y[d] = own.threads_y[d]; p->lpc_y[d] = own.lpc_y[d]; }
+      }
+      p->threads_z = own.threads_z;
+      p->lpc_z = own.lpc_z;
     }
   }
   ~SettingsSwap() {
@@ -1360,7 +1381,7 @@ static int tune_batch(pp_plan* const* plans, int n, cudaStream_t st) {
     float t[2] = {1e30f, 1e30f};
     for (int v = 0; v < 2; v++) {
       SettingsSwap swap;
-      if (v == 1) swap.apply(plans, n);
+      swap.apply(plans, n, v == 1);
       cudaGraphExec_t g = nullptr;
       if (capture_batch(plans, fs.data(), us.data(), n, &g) == PP_OK) {
         t[v] = time_graph(g, st);
@@ -1618,7 +1639,7 @@ pp_status pp_solve_batched(pp_plan* const* plans, const void* const* f, void* co
   pp_status s;
   {
     SettingsSwap swap;
-    if (choice == 1) swap.apply(plans, n);
+    swap.apply(plans, n, choice == 1);
     s = capture_batch(plans, f, u, n, &exec);
   }
   if (s != PP_OK) return s;
