@@ -249,30 +249,7 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
     }
     re = im = df{0.f, 0.f};
   };
-  // The tile one CTA per SM ahead, into L2: a tile's loads then wait for L2 and not for HBM (1024^3 x-forward
-  // 5.95 -> 5.64 ms, y 6.0 -> 5.8, x-inverse 6.8 -> 6.3; 512^3 R2C 0.93 -> 0.78; two or three tiles per SM
-  // ahead: less).  C2C lines, which do the least work per value, lose 2 % to the extra instructions.
-  if constexpr (!C2C) {
-    const unsigned ahead = blockIdx.x + a.ahead;
-    if (ahead < gridDim.x) {
-      if constexpr (!OY) {
-        const unsigned g1 = ahead * NL + (unsigned)L;
-        if (a.vec_ok && lt == 0 && g1 < (unsigned)a.nlines) {  // (16-byte aligned rows of N reals)
-          const SI* q = reinterpret_cast<const SI*>(a.in) + line_base(a, g1, false);
-          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(__cvta_generic_to_global(q)),
-                       "r"((unsigned)(N * (int)sizeof(SI))) : "memory");
-        }
-      } else {
-        const int plane = (int)a.fd_nblk.div(ahead);
-        const int c0 = ((int)ahead - plane * a.nblk) * a.tx;
-        const unsigned g1 = (unsigned)(plane * a.lines_per_plane + c0 * a.parts);
-        const SI* q = reinterpret_cast<const SI*>(a.in) + line_base(a, g1, false);
-        const int rows = C2C ? M : (HG == HG_INV && kind == LK_C2R) ? M + 1 : N;
-        for (int r = tid; r < rows; r += H::T)
-          asm volatile("prefetch.global.L2 [%0];\n" ::"l"(__cvta_generic_to_global(q + (long long)r * ip)));
-      }
-    }
-  }
+  prefetch_tile<SI, OY>(a, blockIdx.x + a.ahead, kind == LK_C2R ? M + 1 : N);
   float mx = 0.0f, l1 = 0.0f;
   // Spill pairs come unnormalised, and a line of cancelled values may hold them in the low parts alone: the
   // leading part becomes the nearest FP32 value of the pair, for the line's scale and the split at it.

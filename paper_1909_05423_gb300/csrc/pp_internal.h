@@ -62,9 +62,14 @@ struct LineArgs {
   const void* haux;
   HScale hs;
   int hdir;
-  int ahead;          // tiles between the one a CTA works on and the one it prefetches into L2
+  int ahead, pf;      // tiles between the one a CTA works on and the one it prefetches into L2; allowed
 };
-constexpr int kHAhead = 152;  // LineArgs::ahead: one tile per SM (pp_hlines.cuh)
+// LineArgs::ahead: one tile per SM.  A tile's loads then wait for L2 and not for HBM (ms without / with; two or
+// more tiles per SM ahead: less or worse).  x lines: block-scaled 1024^3 5.95 / 5.64 forward, 6.8 / 6.3 back,
+// 512^3 R2C 0.93 / 0.78; FP32 1024^3 2.65 / 2.61 and 2.76 / 2.70, 512^3 R2C 0.444 / 0.355, C2R 0.365 / 0.325.
+// y lines: block-scaled real kinds 6.0 / 5.8; FP32 C2C 0.505 / 0.423.  Block-scaled C2C lines lose 2 % and the
+// FP32 real kinds, which batch their loads, 4 %: they do without (LineArgs::pf).
+constexpr int kAhead = 152;
 constexpr int kMaxLpc = 512;  // lines per CTA (bounds the per-line bases in shared memory)
 constexpr int kHostChunks = 8;  // plane chunks of a host-buffer solve (copies overlap transforms)
 

@@ -57,6 +57,28 @@ __device__ __forceinline__ long long line_base(const LineArgs& a, unsigned g, bo
              : (long long)plane * a.in_plane + (long long)c * a.in_line + part;
 }
 
+// Prefetch of tile `tile` into L2 by the whole CTA: x tiles one bulk prefetch per row (a.pf: rows are
+// 16-byte aligned and sized), y tiles one per row of the tile, at its first column.  rows: positions of a y line.
+template <class SI, bool OY>
+__device__ __forceinline__ void prefetch_tile(const LineArgs& a, unsigned tile, int rows) {
+  if (!a.pf || tile >= gridDim.x) return;
+  const SI* in = reinterpret_cast<const SI*>(a.in);
+  if constexpr (!OY) {
+    for (int L = threadIdx.x; L < a.lpc; L += blockDim.x) {
+      const unsigned g = tile * (unsigned)a.lpc + (unsigned)L;
+      if (g < (unsigned)a.nlines)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(__cvta_generic_to_global(in + line_base(a, g, false))),
+                     "r"((unsigned)(a.N * (int)sizeof(SI))) : "memory");
+    }
+  } else {
+    const int plane = (int)a.fd_nblk.div(tile);
+    const int c0 = ((int)tile - plane * a.nblk) * a.tx;
+    const SI* q = in + line_base(a, (unsigned)(plane * a.lines_per_plane + c0 * a.parts), false);
+    for (int r = threadIdx.x; r < rows; r += blockDim.x)
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(__cvta_generic_to_global(q + (long long)r * a.in_pos)));
+  }
+}
+
 // Visit every (line L, item k) of the tile.  x: k fastest (consecutive threads along a line);
 // y: L fastest (consecutive threads across columns).  KC: compile-time item count (0: fdk).
 template <bool OY, int KC, class F>
@@ -912,6 +934,7 @@ __global__ void __maxnreg__((MaxRegs<R, MC, OY>::v)) k_lines(const LineArgs args
     s_bin[L] = line_base(a, (unsigned)(line0 + L), false);
     s_bout[L] = line_base(a, (unsigned)(line0 + L), true);
   }
+  prefetch_tile<SI, OY>(a, blockIdx.x + a.ahead, kind == LK_C2R ? M + 1 : a.N);
   __syncthreads();
   pre_tile<R, OY, MCT>(a, SrcGlobal<R, SI>{reinterpret_cast<const SI*>(a.in), s_bin, (long long)a.in_pos}, nl, buf);
   cp_async_wait_all();

@@ -628,6 +628,7 @@ enum { ST_F64 = 0, ST_F32 = 1, ST_SPILL = 2 };
 
 // division helpers of one launch
 static void finish_args(LineArgs& a) {
+  a.ahead = kAhead;
   int M = a.fp.M, N = a.N, K;
   // Hermitian-pair kinds handle k and M-k in one item, k <= M/2
   switch (a.kind) {
@@ -666,7 +667,6 @@ static void set_hx(LineArgs& a, const void* tab, int dir) {
   a.haux = static_cast<const char*>(tab) + (size_t)a.fp.M * (sizeof(htwa) + sizeof(htwb));
   a.hs = hx_bounds(a.kind, a.fp);
   a.hdir = dir;
-  a.ahead = kHAhead;
 }
 
 // bytes per real of a storage code
@@ -710,6 +710,8 @@ cudaError_t launch_lines(const pp_plan* p, int axis, int dir, int io_in, int io_
     a.ntiles = (a.nlines + a.lpc - 1) / a.lpc;
     a.vec_ok = (((uintptr_t)in | (uintptr_t)out) % 32 == 0) ? 1 : 0;
     a.fd_gpc = FastDiv::make(1u);
+    const size_t se = st_bytes(p, io_in);
+    a.pf = (uintptr_t)in % 16 == 0 && a.N * se % 16 == 0 && a.in_line * se % 16 == 0 && a.in_plane * se % 16 == 0;
     finish_args(a);
     if (p->hx_x[dir]) {
       set_hx(a, p->d_h_x, dir);
@@ -755,6 +757,7 @@ cudaError_t launch_lines(const pp_plan* p, int axis, int dir, int io_in, int io_
   a.ncols = ncols;
   a.nblk = (ncols + a.tx - 1) / a.tx;
   a.ntiles = a.nblk * nzc;
+  a.pf = p->hx_y[dir] != (a.kind == LK_C2C_F || a.kind == LK_C2C_I);
   if (p->hx_y[dir]) {
     a.fd_gpc = FastDiv::make(1u);
     finish_args(a);
@@ -846,6 +849,7 @@ static cudaError_t launch_zlines(const pp_plan* p, int dir, void* data, cudaStre
   a.ncols = (int)ncols;
   a.nblk = (int)((ncols + a.tx - 1) / a.tx);
   a.ntiles = a.nblk;
+  a.pf = !p->hx_z;
   if (p->hx_z) {
     a.fd_gpc = FastDiv::make(1u);
     finish_args(a);
