@@ -209,6 +209,7 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
   const htwb* x1b = reinterpret_cast<const htwb*>(x1a + (M + 2));
   const htwa* x2a = reinterpret_cast<const htwa*>(x1b + (M + 2));
   const htwb* x2b = reinterpret_cast<const htwb*>(x2a + (M + 2));
+  pdl_start();
   for (int i = threadIdx.x; i < MC; i += H::T)
     cp_async_cx(reinterpret_cast<cx<df>*>(sta) + i, reinterpret_cast<const cx<df>*>(gta) + i);
   cp_async_commit();
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
     }
     re = im = df{0.f, 0.f};
   };
+  pdl_wait();
   prefetch_tile<SI, OY>(a, blockIdx.x + a.ahead, kind == LK_C2R ? M + 1 : N);
   float mx = 0.0f, l1 = 0.0f;
   // Spill pairs come unnormalised, and a line of cancelled values may hold them in the low parts alone: the
@@ -600,8 +602,7 @@ cudaError_t launch_hlines_k(const LineArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr_done.fetch_or(bit, std::memory_order_release);
   }
-  k<<<a.ntiles, H::T, H::smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(a.pdl, k, (unsigned)a.ntiles, (unsigned)H::T, H::smem, st, a);
 }
 
 // One translation unit per length (compiled in parallel).

@@ -912,6 +912,7 @@ __global__ void __maxnreg__((MaxRegs<R, MC, OY>::v)) k_lines(const LineArgs args
   long long* s_bin = reinterpret_cast<long long*>(tws + M);
   long long* s_bout = s_bin + a.lpc;
   const cx<R>* twg = reinterpret_cast<const cx<R>*>(a.tw);
+  pdl_start();
   // stage twiddles: w_M^j, j < M (run-time lengths) or the per-stage table of fft_lines_ct.
   // Asynchronous copies (cp.async), waited for after the pre-processing: their latency then
   // overlaps the line loads instead of preceding them.
@@ -934,6 +935,7 @@ __global__ void __maxnreg__((MaxRegs<R, MC, OY>::v)) k_lines(const LineArgs args
     s_bin[L] = line_base(a, (unsigned)(line0 + L), false);
     s_bout[L] = line_base(a, (unsigned)(line0 + L), true);
   }
+  pdl_wait();
   prefetch_tile<SI, OY>(a, blockIdx.x + a.ahead, kind == LK_C2R ? M + 1 : a.N);
   __syncthreads();
   pre_tile<R, OY, MCT>(a, SrcGlobal<R, SI>{reinterpret_cast<const SI*>(a.in), s_bin, (long long)a.in_pos}, nl, buf);
@@ -975,8 +977,7 @@ cudaError_t launch_lines_k(const LineArgs& a, int threads, cudaStream_t st) {
     attr_done.fetch_or(bit, std::memory_order_release);
   }
   const size_t sm = ((size_t)a.lpc * a.ldm + (size_t)a.fp.M) * sizeof(cx<R>) + 2 * (size_t)a.lpc * sizeof(long long);
-  k<<<a.ntiles, threads, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(a.pdl, k, (unsigned)a.ntiles, (unsigned)threads, sm, st, a);
 }
 
 // storage codes of the launchers

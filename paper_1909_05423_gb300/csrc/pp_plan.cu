@@ -677,6 +677,7 @@ cudaError_t launch_lines(const pp_plan* p, int axis, int dir, int io_in, int io_
                          cudaStream_t st, int z0, int nzc) {
   LineArgs a;
   memset(&a, 0, sizeof a);
+  a.pdl = p->pdl;
   if (nzc < 0) { z0 = 0; nzc = p->nz; }
   if (z0 < 0 || nzc < 1 || z0 + nzc > p->nz) return cudaErrorInvalidValue;
   const bool dfm = (p->dtype == PP_F64);
@@ -802,6 +803,7 @@ static void zsolve_args(const pp_plan* p, void* data, int transpose, ZArgs& a) {
   split2(p->zscale, a.scale);
   a.transpose = transpose;
   a.nsing = p->singular ? (a.cplx ? 2 : 1) : 0;
+  a.pdl = p->pdl;
   a.rstat = p->d_status;
   a.dmin = 0x1p-100f;
   a.umax = (float)(0x1p124 / ((double)p->nx * (double)p->ny));
@@ -1212,7 +1214,7 @@ void evict_plan(const pp_plan* p) {
 // Launch settings of a plan that a batched graph may swap: launch shapes and the z algorithm.
 struct PlanSettings {
   int threads_x[2], lpc_x[2], ldm_x, threads_y[2], lpc_y[2], ldm_y, threads_z, lpc_z, ldm_z, zsplit, zmethod;
-  bool hx_x[2], hx_y[2];
+  bool hx_x[2], hx_y[2], pdl;
 };
 static PlanSettings get_settings(const pp_plan* p) {
   PlanSettings s;
@@ -1224,6 +1226,7 @@ static PlanSettings get_settings(const pp_plan* p) {
   s.ldm_x = p->ldm_x; s.ldm_y = p->ldm_y;
   s.threads_z = p->threads_z; s.lpc_z = p->lpc_z; s.ldm_z = p->ldm_z;
   s.zsplit = p->zsplit;
+  s.pdl = p->pdl;
   s.zmethod = p->zmethod;
   return s;
 }
@@ -1236,6 +1239,7 @@ static void set_settings(pp_plan* p, const PlanSettings& s) {
   p->ldm_x = s.ldm_x; p->ldm_y = s.ldm_y;
   p->threads_z = s.threads_z; p->lpc_z = s.lpc_z; p->ldm_z = s.ldm_z;
   p->zsplit = s.zsplit;
+  p->pdl = s.pdl;
   p->zmethod = s.zmethod;
 }
 
@@ -1257,6 +1261,7 @@ struct SettingsSwap {
       if (seen) continue;
       const PlanSettings own = get_settings(p);
       saved.emplace_back(p, own);
+      p->pdl = false;
       for (int d = 0; d < 2; d++) {
         p->hx_x[d] = own.hx_x[d] && p->fx.M >= 256;
         p->hx_y[d] = own.hx_y[d] && p->fy.M >= 256;
@@ -1528,6 +1533,7 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
     p->tuned = true;
     p->z_tuned = zper ? (zreq != 2) : (sreq == 0);
   }
+  p->pdl = true;  // (not for the autotuner's concurrent copies)
   *out = p;
   return PP_OK;
 }

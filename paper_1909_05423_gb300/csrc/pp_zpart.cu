@@ -234,7 +234,9 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
   // of y_0, and c per line
   extern __shared__ float2 zp_sm[];
   float dmax = 0.0f, umax = 0.0f;
+  pdl_start();
   if ((int)blockIdx.x < a.nsing) {
+    pdl_wait();
     zsing_block<S>(a, (int)blockIdx.x, zp_sm, dmax, umax);
     range_report(a.rstat, a.dmin, a.umax, gridDim.x, dmax, umax);
     return;
@@ -266,16 +268,6 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
     }
   }
   const int k0 = c * M;
-  const int nr = max(0, min(M, n - k0));  // rows of the chunk (below M only at the line's end)
-  S* base = reinterpret_cast<S*>(a.data) + s + (long long)k0 * PL;
-  df v[M];
-  if (live && nr == M) {
-#pragma unroll
-    for (int i = 0; i < M; i++) v[i] = zp_ld(base + (long long)i * PL);
-  } else {
-#pragma unroll
-    for (int i = 0; i < M; i++) v[i] = (live && i < nr) ? zp_ld(base + (long long)i * PL) : df{0.f, 0.f};
-  }
   ZpW W;
   W.wt = a.wtab;
   W.wlen = 0;
@@ -292,6 +284,17 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
     W.wt = a.wtab + off.x;
     mine = (m->flags & ZF_NEAR1) != 0;
     if (PER) qlen = off.w;
+  }
+  pdl_wait();
+  const int nr = max(0, min(M, n - k0));  // rows of the chunk (below M only at the line's end)
+  S* base = reinterpret_cast<S*>(a.data) + s + (long long)k0 * PL;
+  df v[M];
+  if (live && nr == M) {
+#pragma unroll
+    for (int i = 0; i < M; i++) v[i] = zp_ld(base + (long long)i * PL);
+  } else {
+#pragma unroll
+    for (int i = 0; i < M; i++) v[i] = (live && i < nr) ? zp_ld(base + (long long)i * PL) : df{0.f, 0.f};
   }
   // a warp runs the near -1 form when any of its modes needs it (the others convert their w); every
   // warp holds all G lines, so all warps of the CTA agree
@@ -433,8 +436,7 @@ static cudaError_t launch_zpart_t(const ZArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr_done.fetch_or(bit, std::memory_order_release);
   }
-  k_zpart<S, M, PER><<<(unsigned)grid, threads, sm, st>>>(a, G, lgG, P);
-  return cudaGetLastError();
+  return launch_pdl(a.pdl, k_zpart<S, M, PER>, (unsigned)grid, (unsigned)threads, sm, st, a, G, lgG, P);
 }
 
 template <class S, bool PER>

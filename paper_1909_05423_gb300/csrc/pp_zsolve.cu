@@ -490,6 +490,8 @@ template <int MODE> struct ZCkMinBlocks { static constexpr int v = (MODE == 1) ?
 template <int MODE>
 __global__ void __launch_bounds__(256, (ZCkMinBlocks<MODE>::v)) k_zsolve_ck(const ZArgs a) {
   float dmax = 0.0f, umax = 0.0f;
+  pdl_start();
+  pdl_wait();
   __shared__ float2 sm[kZsingSmem / sizeof(float2)];
   if ((int)blockIdx.x < a.nsing) zsing_block<float2>(a, (int)blockIdx.x, sm, dmax, umax);
   else z_line_ck<MODE>(a, dmax, umax);
@@ -499,6 +501,8 @@ __global__ void __launch_bounds__(256, (ZCkMinBlocks<MODE>::v)) k_zsolve_ck(cons
 template <class S, int MODE>
 __global__ void __launch_bounds__(256, (ZMinBlocks<S, MODE>::v)) k_zsolve(const ZArgs a) {
   float dmax = 0.0f, umax = 0.0f;
+  pdl_start();
+  pdl_wait();
   __shared__ float2 sm[kZsingSmem / sizeof(float2)];
   if ((int)blockIdx.x < a.nsing) zsing_block<S>(a, (int)blockIdx.x, sm, dmax, umax);
   else z_line<S, MODE>(a, dmax, umax);
@@ -507,10 +511,8 @@ __global__ void __launch_bounds__(256, (ZMinBlocks<S, MODE>::v)) k_zsolve(const 
 
 template <class S>
 static cudaError_t launch_z(const ZArgs& a, int mode, unsigned grid, int threads, cudaStream_t st) {
-  if (mode == 1) k_zsolve<S, 1><<<grid, threads, 0, st>>>(a);
-  else if (mode == 2) k_zsolve<S, 2><<<grid, threads, 0, st>>>(a);
-  else k_zsolve<S, 0><<<grid, threads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(a.pdl, mode == 1 ? k_zsolve<S, 1> : mode == 2 ? k_zsolve<S, 2> : k_zsolve<S, 0>, grid, (unsigned)threads,
+                    (size_t)0, st, a);
 }
 
 cudaError_t launch_zsolve_impl(const ZArgs& a, bool df_spill, bool zper, cudaStream_t st) {
@@ -521,10 +523,8 @@ cudaError_t launch_zsolve_impl(const ZArgs& a, bool df_spill, bool zper, cudaStr
   if (df_spill) {
     // the double-float spill always runs the checkpointed sweeps (they need the checkpoint buffer)
     if (!a.ck) return cudaErrorInvalidValue;
-    if (mode == 1) k_zsolve_ck<1><<<(unsigned)grid, threads, 0, st>>>(a);
-    else if (mode == 2) k_zsolve_ck<2><<<(unsigned)grid, threads, 0, st>>>(a);
-    else k_zsolve_ck<0><<<(unsigned)grid, threads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(a.pdl, mode == 1 ? k_zsolve_ck<1> : mode == 2 ? k_zsolve_ck<2> : k_zsolve_ck<0>, (unsigned)grid,
+                      (unsigned)threads, (size_t)0, st, a);
   }
   return launch_z<float>(a, mode, (unsigned)grid, threads, st);
 }

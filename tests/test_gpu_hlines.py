@@ -91,3 +91,23 @@ def test_non_finite_source(bad):
     assert e.value.status == _lib.PP_ERR_RANGE
     assert not torch.isfinite(u[2]).any()
     plan.close()
+
+
+def test_solve_inside_a_captured_graph():
+    """The overlapped launches of a small grid record into a caller's graph and replay on new data."""
+    import paper_1909_05423_gb300 as pp
+    shape = (20, 24, 64)
+    plan = pp.Plan(shape, "NNPPND", (1.0 / 64,) * 3, "f64")
+    f, u = (torch.zeros(shape, dtype=torch.float64, device="cuda") for _ in range(2))
+    plan.solve(f, out=u)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        plan.solve(f, out=u, stream=torch.cuda.current_stream())
+        plan.solve(u, out=u, stream=torch.cuda.current_stream())
+    for seed in range(3):
+        f.copy_(torch.from_numpy(workloads.uniform_source(shape, seed=90 + seed)))
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(u, plan.solve(plan.solve(f)))
+    plan.close()
