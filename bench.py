@@ -64,7 +64,8 @@ KERNEL_SOURCES = ("pp_arith.cuh", "pp_fft.cuh", "pp_internal.h", "pp_lines.cuh",
                   "pp_lines_df_large.cu", "pp_lines_df_any.cu", "pp_lines_df_any57.cu", "pp_lines_f32_small.cu",
                   "pp_lines_f32_large.cu", "pp_lines_f32_any.cu", "pp_lines_f32_any57.cu", "pp_lines_df_ct3a.cu",
                   "pp_lines_df_ct3b.cu", "pp_lines_f32_ct3a.cu", "pp_lines_f32_ct3b.cu", "pp_zsolve.cu", "pp_zpart.cu",
-                  "pp_zfft.cu", "pp_range.cuh", "pp_zmul.cuh")
+                  "pp_zfft.cu", "pp_range.cuh", "pp_zmul.cuh", "pp_zsing.cuh", "pp_hx.cuh", "pp_hlines.cuh",
+                  "pp_hlines_64.cu", "pp_hlines_128.cu", "pp_hlines_256.cu", "pp_hlines_512.cu", "pp_hlines_1024.cu")
 
 
 def _code_only(text: str) -> str:
@@ -105,14 +106,18 @@ def _traffic(stage: str, n: int):
 # double-float in the unnormalised forms the line kernels use: add 8 (TwoSum 6, two lo adds),
 # multiply 4 (FMUL, 3 FFMA), complex multiply 32 (two fused a*b -+ c*d of 16: two TwoProds 4,
 # TwoSum 6, 6 adds and FMAs of the error terms), complex add 16, halving 2; FP32: add 1, multiply 1,
-# complex multiply 4, complex add 2.  Peak: 152 SMs x 128 FP32 lanes x 2.07 GHz (maximum SM clock).
+# complex multiply 4, complex add 2.  Block-scaled integer + float values (the FP64-class kernels of
+# power-of-two lengths, pp_hx.cuh): issue slots as measured for chains in registers, add 2 (one integer, one
+# float), complex multiply 38 and product with 1/sqrt 2 15 (a 32 x 32 -> 64-bit multiply-add takes 5.2), the
+# quarter beside a product 8.  Peak: 152 SMs x 128 FP32 lanes x 2.07 GHz (maximum SM clock).
 FP32_LANES = 152 * 128
 SM_MAX_GHZ = 2.07
-_OPS = {"df": {"add": 8, "mul": 4, "cmul": 32, "half": 2}, "f32": {"add": 1, "mul": 1, "cmul": 4, "half": 1}}
+_OPS = {"df": {"add": 8, "mul": 4, "cmul": 32, "half": 2}, "f32": {"add": 1, "mul": 1, "cmul": 4, "half": 1},
+        "hx": {"add": 2, "mul": 15, "cmul": 38, "half": 8}}
 
 
 def fft_ops(M: int, arith: str) -> float:
-    """FP32 operations of one complex FFT of power-of-two length M (radix 8, then 4 or 2; the last
+    """Lane instructions of one complex FFT of power-of-two length M (radix 8, then 4 or 2; the last
     stage has no twiddles)."""
     o = _OPS[arith]
     cadd = 2 * o["add"]
@@ -130,7 +135,7 @@ def fft_ops(M: int, arith: str) -> float:
 
 
 def line_ops_per_real(kind: str, N: int, arith: str) -> float:
-    """FP32 operations per real point of one real line transform of length N (complex FFT of N/2
+    """Lane instructions per real point of one real line transform of length N (complex FFT of N/2
     points plus the pre/post-processing of the kind): DCT-II/DST-II (Hermitian-pair split and
     the quarter-wave twiddle), DCT-III/DST-III (the reverse), as implemented."""
     o = _OPS[arith]
@@ -645,7 +650,8 @@ def run_ours(args):
     peak, peak_kind = _peaks()
     achieved = alg_bytes[dname] / (per[dom] * 1e-3) / 1e9
     path_gbs = 32.0 * npts / (ms * 1e-3) / 1e9
-    # the line kernels are bound by FP32 instruction issue (double-float arithmetic): ALU roofline
+    # the line kernels are bound by load latency and instruction issue: the issue slots of their arithmetic
+    # (block-scaled where the length has such a kernel, otherwise double-float) beside the HBM fraction
     kinds = {"x-forward": "dct2", "y-forward": "dct2", "y-inverse": "dct3", "x-inverse": "dct3"}  # NN-x, DD-y
     alu_peak = FP32_LANES * SM_MAX_GHZ * 1e9 / 1e12
     per_stage = {}
@@ -653,24 +659,26 @@ def run_ours(args):
         d = {"ms": per[k], "hbm_gbs": alg_bytes[name] / (per[k] * 1e-3) / 1e9}
         d["hbm_frac"] = d["hbm_gbs"] / peak
         if name in kinds:
-            opr = line_ops_per_real(kinds[name], nx_ if name[0] == "x" else ny_, "df")
+            N = nx_ if name[0] == "x" else ny_
+            d["arith"] = "hx" if N & (N - 1) == 0 and 128 <= N <= 2048 else "df"
+            opr = line_ops_per_real(kinds[name], N, d["arith"])
             d["fp32_ops_per_point"] = opr
             d["alu_tops"] = opr * npts / (per[k] * 1e-3) / 1e12
             d["alu_frac"] = d["alu_tops"] / alu_peak
         per_stage[name] = d
     # the roofline block is the dominant kernel's HBM fraction (algorithmic bytes of that launch over
     # its CUDA-event time, against the measured copy bandwidth); the line kernels are in fact bound by
-    # FP32 instruction issue in double-float arithmetic, so that fraction is reported beside it
+    # load latency and instruction issue, so the issue fraction is reported beside it
     roof = {"bound": "hbm", "kernel": dname, "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs, copy bandwidth)" % peak_kind,
             "traffic": None if args.shape else _traffic(dname, n), "alg_bytes_per_launch": alg_bytes[dname],
             "alg_bytes_per_point": alg_bytes[dname] / npts}
     if dname in kinds:
         roof["alu"] = {"achieved": per_stage[dname]["alu_tops"], "peak": alu_peak,
-                       "unit": "T FP32 lane instructions/s", "frac": per_stage[dname]["alu_frac"],
+                       "unit": "T lane instructions/s", "frac": per_stage[dname]["alu_frac"],
                        "alg_fp32_instr_per_point": per_stage[dname]["fp32_ops_per_point"],
-                       "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz; algorithmic double-float "
-                                      "operations counted as the FP32 lane instructions they issue (FMA = 1)"}
+                       "peak_source": "derived: 152 SMs x 128 lanes x 2.07 GHz; algorithmic operations counted as "
+                                      "the issue slots they take (arith: %s)" % per_stage[dname]["arith"]}
 
     # ---------------------------------------------------------------- mixed precision variants
     variants = {}
