@@ -96,7 +96,9 @@ struct LineArgs {
 // more tiles per SM ahead: less or worse).  x lines: block-scaled 1024^3 5.95 / 5.64 forward, 6.8 / 6.3 back,
 // 512^3 R2C 0.93 / 0.78; FP32 1024^3 2.65 / 2.61 and 2.76 / 2.70, 512^3 R2C 0.444 / 0.355, C2R 0.365 / 0.325.
 // y lines: block-scaled real kinds 6.0 / 5.8; FP32 C2C 0.505 / 0.423.  Block-scaled C2C lines lose 2 % and the
-// FP32 real kinds, which batch their loads, 4 %: they do without (LineArgs::pf).
+// FP32 real kinds, which batch their loads, 4 %: they do without (LineArgs::pf).  So do the z lines of the z
+// transform, whose tiles take one sector of every plane: mixed, all-periodic 27.0 / 30.5 for the 1024^3 solve, 3.07 /
+// 2.95 at 512^3, 0.413 / 0.417 at 256^3.
 constexpr int kAhead = 152;
 constexpr int kMaxLpc = 512;  // lines per CTA (bounds the per-line bases in shared memory)
 constexpr int kHostChunks = 8;  // plane chunks of a host-buffer solve (copies overlap transforms)

@@ -851,7 +851,7 @@ static cudaError_t launch_zlines(const pp_plan* p, int dir, void* data, cudaStre
   a.ncols = (int)ncols;
   a.nblk = (int)((ncols + a.tx - 1) / a.tx);
   a.ntiles = a.nblk;
-  a.pf = !p->hx_z;
+  a.pf = 0;  // see kAhead
   if (p->hx_z) {
     a.fd_gpc = FastDiv::make(1u);
     finish_args(a);
