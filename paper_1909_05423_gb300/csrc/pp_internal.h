@@ -17,7 +17,8 @@ namespace pp {
 // latency and prologues where a kernel is short: 32^3 alone 65.6 -> 58.9 us (back to back the host's launches
 // bound it), 120 x 140 x 99 167 -> 158 us.  Grids of more than 16 CTAs per SM are launched plainly: the CTAs
 // that start early hold room that the kernel before them still wants (256^3 535 -> 548 us, 1024^3 27.3 -> 30.5
-// ms).  So are the members of a batch graph, where other branches want that room (64 grids 2.88 -> 2.92 ms).
+// ms).  So are the members of a batch graph, where other branches want that room (64 grids 2.88 -> 2.92 ms), and the
+// z sweeps (pp_zsolve.cu).
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 constexpr unsigned kPdlGrid = 16 * 152;

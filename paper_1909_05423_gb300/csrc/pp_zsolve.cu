@@ -487,11 +487,12 @@ __device__ __forceinline__ void z_line_ck(const ZArgs& a, float& dmax, float& um
 // at 3 CTAs without spills, measured), 3 for the cyclic sweeps (they would spill 300 bytes at 64)
 template <int MODE> struct ZCkMinBlocks { static constexpr int v = (MODE == 1) ? 3 : 4; };
 
+// The sweeps are launched plainly (pp_internal.h, launch_pdl): CTAs that start while the y-forward drains gather
+// on the few SMs with room, and few lines then share an SM's issue instead of having one each (solve in sweeps of
+// 4095 x 64 x 64 4.84 -> 5.04 ms, mixed adjoint of 128^3 0.122 -> 0.135 ms).
 template <int MODE>
 __global__ void __launch_bounds__(256, (ZCkMinBlocks<MODE>::v)) k_zsolve_ck(const ZArgs a) {
   float dmax = 0.0f, umax = 0.0f;
-  pdl_start();
-  pdl_wait();
   __shared__ float2 sm[kZsingSmem / sizeof(float2)];
   if ((int)blockIdx.x < a.nsing) zsing_block<float2>(a, (int)blockIdx.x, sm, dmax, umax);
   else z_line_ck<MODE>(a, dmax, umax);
@@ -501,8 +502,6 @@ __global__ void __launch_bounds__(256, (ZCkMinBlocks<MODE>::v)) k_zsolve_ck(cons
 template <class S, int MODE>
 __global__ void __launch_bounds__(256, (ZMinBlocks<S, MODE>::v)) k_zsolve(const ZArgs a) {
   float dmax = 0.0f, umax = 0.0f;
-  pdl_start();
-  pdl_wait();
   __shared__ float2 sm[kZsingSmem / sizeof(float2)];
   if ((int)blockIdx.x < a.nsing) zsing_block<S>(a, (int)blockIdx.x, sm, dmax, umax);
   else z_line<S, MODE>(a, dmax, umax);
@@ -511,8 +510,10 @@ __global__ void __launch_bounds__(256, (ZMinBlocks<S, MODE>::v)) k_zsolve(const 
 
 template <class S>
 static cudaError_t launch_z(const ZArgs& a, int mode, unsigned grid, int threads, cudaStream_t st) {
-  return launch_pdl(a.pdl, mode == 1 ? k_zsolve<S, 1> : mode == 2 ? k_zsolve<S, 2> : k_zsolve<S, 0>, grid, (unsigned)threads,
-                    (size_t)0, st, a);
+  if (mode == 1) k_zsolve<S, 1><<<grid, threads, 0, st>>>(a);
+  else if (mode == 2) k_zsolve<S, 2><<<grid, threads, 0, st>>>(a);
+  else k_zsolve<S, 0><<<grid, threads, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_zsolve_impl(const ZArgs& a, bool df_spill, bool zper, cudaStream_t st) {
@@ -523,8 +524,10 @@ cudaError_t launch_zsolve_impl(const ZArgs& a, bool df_spill, bool zper, cudaStr
   if (df_spill) {
     // the double-float spill always runs the checkpointed sweeps (they need the checkpoint buffer)
     if (!a.ck) return cudaErrorInvalidValue;
-    return launch_pdl(a.pdl, mode == 1 ? k_zsolve_ck<1> : mode == 2 ? k_zsolve_ck<2> : k_zsolve_ck<0>, (unsigned)grid,
-                      (unsigned)threads, (size_t)0, st, a);
+    if (mode == 1) k_zsolve_ck<1><<<(unsigned)grid, threads, 0, st>>>(a);
+    else if (mode == 2) k_zsolve_ck<2><<<(unsigned)grid, threads, 0, st>>>(a);
+    else k_zsolve_ck<0><<<(unsigned)grid, threads, 0, st>>>(a);
+    return cudaGetLastError();
   }
   return launch_z<float>(a, mode, (unsigned)grid, threads, st);
 }
