@@ -927,15 +927,27 @@ static pp_status run_stage(pp_plan* p, int stage, const void* f, void* u, int tr
 //          periodic z: 192^3 0.246/0.076/0.082   512^3 1.162/1.126/1.163
 //   mixed  256 x 320^2 0.240/0.156/0.137   256 x 448^2 0.299/0.301/0.262   64 x 512^2 0.092/0.113/0.105
 //          512^3 0.61/0.83/0.67   periodic z: 256^3 0.274/0.133/0.145
+// and on longer lines (sweeps / 16 rows):
+//   FP64   300 x 448 x 512 0.477/0.435   600 x 448 x 512 0.914/0.917   800 x 256 x 448 0.948/0.635
+//          1138 x 224 x 448 1.214/1.040   1138 x 288 x 512 1.425/1.534   1138 x 448 x 512 1.571/2.387
+//   mixed  300 x 384^2 0.296/0.253   300 x 448 x 512 0.375/0.388   420 x 320 x 512 0.419/0.394
+//          600 x 384^2 0.534/0.629   1138 x 160 x 512 0.700/0.741   1138 x 288 x 512 0.981/1.350
+//          periodic z, 8 rows: 1138 x 288 x 512 1.49/2.37
 // The sweeps read and write at the copy bandwidth once their threads (one per real slot) fill the GPU;
 // below that a line's serial chain sets their time, whatever the number of lines.  The partitioned solve
-// does 1.5 times their arithmetic and takes 6 ps a value.  The lines cross near 290 k slots for the
-// double-float spill (checkpointed sweeps) and 230 k for FP32.  16 rows a chunk do less carry work, 8
-// give twice the threads: worth it up to 8 M values, and for periodic z, whose q terms weigh on the
-// first chunks.
+// does 1.5 times their arithmetic and takes 6 ps a value, up to 9 where a CTA of long lines leaves
+// much of an SM's threads idle.  So the number of slots at which the two cross falls with the rows, and
+// is lower for the FP32 spill, whose sweeps move less; the steps below stay under it.  16 rows a chunk do
+// less carry work, 8 give twice the threads: worth it up to 8 M values, and for periodic z, whose q terms
+// weigh on the first chunks.
 static int z_rows_default(const pp_plan* p) {
   const bool zper = p->bc[4] == PP_BC_PERIODIC;
-  if (p->splane > (p->dtype == PP_F64 ? 290000 : 230000)) return 1;
+  const bool f64 = p->dtype == PP_F64;
+  long long most;  // slots
+  if (zper) most = p->nz > 512 ? 110000 : f64 ? 290000 : 230000;
+  else if (f64) most = p->nz <= 300 ? 290000 : p->nz <= 600 ? 200000 : 90000;
+  else most = p->nz <= 300 ? 200000 : p->nz <= 450 ? 160000 : 60000;
+  if (p->splane > most) return 1;
   int M = (zper || p->splane * p->nz <= (8LL << 20)) ? 8 : 16;
   int G, lgG, P;
   for (; M <= 32; M *= 2)
