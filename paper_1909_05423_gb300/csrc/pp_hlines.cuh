@@ -261,8 +261,7 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
       v.lo = __fsub_rn(v.lo, __fsub_rn(t, v.hi));
       v.hi = t;
     }
-    mx = fmaxf(mx, fabsf(v.hi));
-    l1 += fabsf(v.hi);
+    hx_stat(mx, l1, v.hi);
   };
   hcx v[16];
   float S;

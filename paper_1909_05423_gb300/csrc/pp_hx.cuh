@@ -8,17 +8,21 @@
 // product with a twiddle takes one 32 x 32 -> 64-bit multiply-add per real product for the integer parts
 // and float FMAs for the rest.
 //
-// Scale.  The transforms are sums of unit-modulus multiples of a line's values, so every intermediate is
-// bounded by the sum of magnitudes l1 of the line, and after s stages by (product of their radices) x
-// sqrt 2 x the largest magnitude.  Every twiddle product is scaled by 1/4, which leaves room for most of
-// a stage's growth.  The scale is the largest power of two that keeps every stage's integers within 0.95
-// 2^31 by one of the two bounds; random lines then start near 2^26 and end near 2^25, a line with a single
+// Scale.  The transforms are sums of unit-modulus multiples of a line's values, so the modulus of every
+// intermediate is bounded by the sum of magnitudes l1 of the line, and after s stages by (product of their
+// radices) x sqrt 2 x the largest magnitude.  The butterflies also form re + im and re - im (hrot8), which reach
+// sqrt 2 times the modulus; hx_bounds says where that counts.  Every twiddle product is scaled by 1/4, which
+// leaves room for most of a stage's growth.  The scale is the largest power of two that keeps every stage's
+// integers within 0.95 2^31 by one of the two bounds; random lines then start near 2^26 and end near 2^25, a line with a single
 // coefficient starts near 2^30, and the rounding of l (2^-25 of a unit) is 2^-49 to 2^-51 of the values;
 // the unnormalised double-float pairs round their low parts at 2^-47.
 //
 // A line with a non-finite value becomes NaN as a whole (every output of a transform depends on every
 // input).
 #pragma once
+#include <algorithm>
+#include <cmath>
+
 #include "pp_arith.cuh"
 
 namespace pp {
@@ -47,6 +51,13 @@ struct alignas(16) htwa {
 struct alignas(8) htwb {
   float c1, s1;
 };
+
+// (host) +-1 as +-(2^30 - 1): products with 2^30 would end in ties, whose remainders have a mean (hquarter)
+inline void hx_twiddle(double c, double s, htwa& a, htwb& b) {
+  auto ints = [](double x) { return (int)std::max(-1073741823LL, std::min(1073741823LL, std::llround(x * 0x1p30))); };
+  a = htwa{ints(c), ints(s), (float)(0.25 * c), (float)(0.25 * s)};
+  b = htwb{(float)(0.25 * (c - a.c * 0x1p-30)), (float)(0.25 * (s - a.s * 0x1p-30))};
+}
 
 // The 64-bit sum rounded to its top word, and the signed remainder beside the float terms u.
 __device__ __forceinline__ hx hx_fin(long long s, float u) {
@@ -175,6 +186,43 @@ struct HScale {
   int n;
   int out;             // exponent of the scale that the products took off
 };
+// (host) Bounds of one transform: every intermediate, per unit of the line's largest magnitude and of its sum
+// of magnitudes, and the factors of 1/4 that the products take off.  iv: type IV; inv: C2R, DCT-III, DST-III;
+// c2c; none of them: R2C, DCT-II, DST-II.  rad: the radices of the nst stages.
+inline HScale hx_bounds(bool iv, bool inv, bool c2c, const int* rad, int nst) {
+  HScale b = {};
+  auto add = [&](double per_max, double per_sum) {
+    b.am[b.n] = (float)(0.95 * 0x1p31 / per_max);
+    b.as[b.n] = (float)(0.95 * 0x1p31 / per_sum);
+    b.n++;
+  };
+  // before the first stage: the values themselves (type IV), sums of two pairs (inverse kinds)
+  if (iv) add(1.0, 1.0);
+  if (inv) add(2.5, 1.0);
+  // In stage s: complex sums of R values of modulus <= sqrt 2 (after the pre-products / 4: type IV), and re +- im of
+  // sums of R/2 of them.  By the sum of magnitudes: l1 bounds |re| + |im| of any sum of a line's own values, so
+  // re +- im too (first stage of C2C and the forward kinds); once a twiddle has turned them it bounds the modulus,
+  // and re +- im reach sqrt 2 l1.  (The pre-products of the inverse kinds turn theirs as well, but with
+  // |E|^2 + |O|^2 = (|A|^2 + |B|^2) / 8 the two values of an item, E +- iO, have moduli of (|A| + |B|) / sqrt 2 at most
+  // together.)
+  double R = 1.0, off = iv ? 0.25 : 1.0;
+  for (int s = 0; s < nst; s++) {
+    R *= rad[s];
+    // (the Hermitian split of the forward kinds adds two of the last stage's results)
+    const double two = (s + 1 == nst && !iv && !inv && !c2c) ? 2.0 : 1.0;
+    const double turned = (iv || (s > 0 && !inv)) ? std::sqrt(2.0) : 1.0;
+    add(two * std::sqrt(2.0) * R * off, std::max(two, turned) * off);
+    if (s + 1 < nst) off *= 0.25;
+  }
+  // products by 1/4: nst - 1 twiddled stages; the pre- and post-products; the forward split works with
+  // twice the even and odd parts
+  b.out = 2 * (nst - 1) + (iv ? 4 : inv ? 2 : c2c ? 0 : 1);
+  return b;
+}
+__device__ __forceinline__ void hx_stat(float& mx, float& l1, float v) {
+  mx = fmaxf(mx, fabsf(v));
+  l1 += fabsf(v);
+}
 __device__ __forceinline__ float hx_scale(const HScale& b, float mx, float l1) {
   const float rm = __frcp_rn(mx), rl = __frcp_rn(l1);
   float s = 0x1p126f;

@@ -263,17 +263,15 @@ static pp_status hx_tables(int ax, int N, bool complex_data, const FftPlan& fp, 
   std::vector<float> v;
   auto bits = [](int x) { float f; memcpy(&f, &x, 4); return f; };
   auto emit = [&](const std::vector<std::pair<double, double>>& w) {
-    // +-1 as +-(2^30 - 1): products with 2^30 would end in ties, whose remainders have a mean (pp_hx.cuh)
-    auto ints = [](double x) { return (int)std::max(-1073741823LL, std::min(1073741823LL, std::llround(x * 0x1p30))); };
+    htwa a;
+    htwb b;
     for (const auto& z : w) {
-      v.push_back(bits(ints(z.first)));
-      v.push_back(bits(ints(z.second)));
-      v.push_back((float)(0.25 * z.first));
-      v.push_back((float)(0.25 * z.second));
+      hx_twiddle(z.first, z.second, a, b);
+      for (float x : {bits(a.c), bits(a.s), a.c0, a.s0}) v.push_back(x);
     }
     for (const auto& z : w) {
-      v.push_back((float)(0.25 * (z.first - ints(z.first) * 0x1p-30)));
-      v.push_back((float)(0.25 * (z.second - ints(z.second) * 0x1p-30)));
+      hx_twiddle(z.first, z.second, a, b);
+      for (float x : {b.c1, b.s1}) v.push_back(x);
     }
   };
   auto e = [](long long num, long long den) {
@@ -301,37 +299,6 @@ static pp_status hx_tables(int ax, int N, bool complex_data, const FftPlan& fp, 
   emit(a1);
   emit(a2);
   return upload(dptr, v);
-}
-
-// Bounds of the block-scaled arithmetic for one transform (pp_hx.cuh): every intermediate, per unit of the
-// line's largest magnitude and of its sum of magnitudes, and the factors of 1/4 that the products take off.
-static HScale hx_bounds(int kind, const FftPlan& fp) {
-  HScale b;
-  memset(&b, 0, sizeof b);
-  auto add = [&](double per_max, double per_sum) {
-    b.am[b.n] = (float)(0.95 * 0x1p31 / per_max);
-    b.as[b.n] = (float)(0.95 * 0x1p31 / per_sum);
-    b.n++;
-  };
-  const bool iv = (kind == LK_DCT4 || kind == LK_DST4);
-  const bool inv = (kind == LK_C2R || kind == LK_DCT3 || kind == LK_DST3);
-  // before the first stage: the values themselves (type IV), sums of two pairs (inverse kinds)
-  if (iv) add(1.0, 1.0);
-  if (inv) add(2.5, 1.0);
-  // after stage s: complex sums of R values of modulus <= sqrt 2 (after the pre-products / 4: type IV)
-  double R = 1.0, off = iv ? 0.25 : 1.0;
-  for (int s = 0; s < fp.nst; s++) {
-    R *= fp.rad[s];
-    // (the Hermitian split of the forward kinds adds two of the last stage's results)
-    const double two = (s + 1 == fp.nst && !iv && !inv && kind != LK_C2C_F && kind != LK_C2C_I) ? 2.0 : 1.0;
-    add(two * std::sqrt(2.0) * R * off, two * off);
-    if (s + 1 < fp.nst) off *= 0.25;
-  }
-  // products by 1/4: nst - 1 twiddled stages; the pre- and post-products; the forward split works with
-  // twice the even and odd parts
-  const int q = 2 * (fp.nst - 1);
-  b.out = q + (iv ? 4 : inv ? 2 : (kind == LK_C2C_F || kind == LK_C2C_I) ? 0 : 1);
-  return b;
 }
 
 // Thomas multipliers of one z system, w_k = h2 / m_k with m_0 = b_0, m_k = b_k - h2 w_{k-1}
@@ -665,7 +632,8 @@ static void set_vec_complex(LineArgs& a, bool dfm, const void* in, const void* o
 static void set_hx(LineArgs& a, const void* tab, int dir) {
   a.htab = tab;
   a.haux = static_cast<const char*>(tab) + (size_t)a.fp.M * (sizeof(htwa) + sizeof(htwb));
-  a.hs = hx_bounds(a.kind, a.fp);
+  a.hs = hx_bounds(a.kind == LK_DCT4 || a.kind == LK_DST4, a.kind == LK_C2R || a.kind == LK_DCT3 || a.kind == LK_DST3,
+                   a.kind == LK_C2C_F || a.kind == LK_C2C_I, a.fp.rad, a.fp.nst);
   a.hdir = dir;
 }
 

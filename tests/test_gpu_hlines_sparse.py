@@ -1,0 +1,72 @@
+"""The scale of the block-scaled line kernels on lines of a few cells, whose sum of magnitudes sets it, through whole
+solves against the oracle (1e-12 relative L2, the tolerance of the FP64-class path).  Every plane holds the same line
+at another magnitude between 1 and 2: the scale is a power of two, so a line can leave its integers at some
+magnitudes only."""
+import numpy as np
+import pytest
+
+from tests.gpu_common import gpu_solve, need_gpu, rel_l2
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-12
+MAGS = tuple(1.0 + k / 24.0 for k in range(24))
+SP = (0.1, 0.1, 0.1)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _setup(oracle):
+    need_gpu()
+
+
+def _planes(line, across):
+    """[plane, ny, nx]: MAGS[plane] x line[i] across[j], the line along x."""
+    return np.array(MAGS)[:, None, None] * across[None, :, None] * line[None, None, :]
+
+
+@pytest.mark.parametrize("n", [128, 512, 2048])
+@pytest.mark.parametrize("kind", ["DN", "ND"])
+def test_four_cells_type_iv(oracle, n, kind):
+    """Cells that meet in one butterfly of the first stage, after the pre-products turned them."""
+    for cells in ((5 * n // 8 - 1, 5 * n // 8, 7 * n // 8 - 1, 7 * n // 8), (n // 8 - 1, n // 8, 3 * n // 8 - 1, 3 * n // 8)):
+        line = np.zeros(n)
+        line[list(cells)] = 1.0
+        f = _planes(line, np.array([1.0, -0.5, 0.25, 2.0]))
+        bc = kind + "NNDD"
+        assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, bc
+        f = np.ascontiguousarray(_planes(line, np.linspace(0.6, 1.7, 6)).transpose(0, 2, 1))
+        bc = "NN" + kind + "DD"
+        assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, bc
+
+
+def _aligned(M, j):
+    """32 complex points that add up at 45 degrees in the second result of the odd half of butterfly j of the second
+    stage (radices 8 and 8), each with the larger of its parts at 1."""
+    t, z = j % 8, np.zeros(M, dtype=complex)
+    for u, c in ((1, 1), (5, -1), (3, -1j), (7, 1j)):
+        for v in range(8):
+            n = j // 8 + u * (M // 64) + v * (M // 8)
+            w = c * np.exp(-2j * np.pi * ((j // 8 + u * (M // 64)) * t % M) / M) * np.exp(-2j * np.pi * (v * t % 8) / 8)
+            x = np.conj(w) * np.exp(0.25j * np.pi)
+            z[n] = x / max(abs(x.real), abs(x.imag))
+    return z
+
+
+@pytest.mark.parametrize("M", [64, 512])
+@pytest.mark.parametrize("j", [1, 5])
+def test_aligned_second_stage(oracle, M, j):
+    z = _aligned(M, j)
+    nx = 8
+    # complex columns: a real source whose x transform is z in column 1
+    f = np.real(z[None, :, None] * np.exp(2j * np.pi * np.arange(nx) / nx)[None, None, :]) * (2.0 / nx)
+    f = np.array(MAGS)[:, None, None] * f
+    assert rel_l2(gpu_solve(f, "PPPPDD", SP), oracle.solve(f, "PPPPDD", SP)) <= TOL
+    # real lines of 2M cells: R2C pairs (u_2k, u_2k+1), the Makhoul order of DCT-II and DST-II
+    r2c = np.empty(2 * M)
+    r2c[0::2], r2c[1::2] = z.real, z.imag
+    mk = np.empty(2 * M)
+    k = np.arange(M // 2)
+    mk[4 * k], mk[4 * k + 2] = z[k].real, z[k].imag
+    mk[4 * k + 3], mk[4 * k + 1] = z[M - 1 - k].real, z[M - 1 - k].imag
+    for line, bc in ((r2c, "PP"), (mk, "NN"), (np.where(np.arange(2 * M) % 2, -mk, mk), "DD")):
+        f = _planes(line, np.array([1.0, -0.5]))
+        assert rel_l2(gpu_solve(f, bc + "NNDD", SP), oracle.solve(f, bc + "NNDD", SP)) <= TOL, bc
