@@ -411,8 +411,12 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
     for (int i = 0; i < 8; i++)
 #pragma unroll
       for (int c = 0; c < 4; c++) stat(r[i][c]);
-    stat(rm[0]);
-    stat(rm[1]);
+    // (the middle item takes its two values as both of its pairs: they count twice)
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      stat(rm[c]);
+      hx_stat(mx, l1, rm[c].hi);
+    }
     h_line_stats<OY, MC>(mx, l1, red, L);
     S = hx_scale(a.hs, mx, l1);
     // E = X_k + conj X_{M-k}, O = (X_k - conj X_{M-k}) conj(w_N^k), both / 4; Z_k = E + i O, Z_{M-k} its

@@ -121,7 +121,7 @@ static Vec transform(int kind, int N, const Vec& in, const Tables& t) {
       if (kind == C2R) {
         y[0] = in[2 * k];
         y[1] = k ? in[2 * k + 1] : 0.0;
-        y[2] = in[2 * (M - k)];
+        y[2] = in[2 * (M - k)];  // (k = M/2: the same two values once more)
         y[3] = k ? in[2 * (M - k) + 1] : 0.0;
       } else {
         auto row = [&](int j) { return in[kind == DCT3 ? j : N - 1 - j]; };
@@ -131,10 +131,6 @@ static Vec transform(int kind, int N, const Vec& in, const Tables& t) {
         y[3] = row(M + k);
       }
       for (int c = 0; c < 4; c++) {
-        if (k == M / 2 && c >= 2) {  // the middle item: its two values, once
-          it[k].y[c] = it[k].y[c - 2];
-          continue;
-        }
         it[k].y[c] = stat(st, y[c]);
       }
     }
@@ -444,6 +440,21 @@ int main(int argc, char** argv) {
           }
         }
       }
+    } else if (fam == "modes") {
+      // one coefficient (a source of a single wave), or two, at the ends and in the middle
+      for (int i : {0, 1, 2, 3, M / 4, M / 2 - 1, M / 2, M / 2 + 1, M - 2, M - 1, M, M + 1, 3 * M / 2 - 1, 3 * M / 2, N - 2, N - 1, reals - 2, reals - 1})
+        for (double m : mags) {
+          if (i < 0 || i >= reals) continue;
+          zero();
+          v[i] = m;
+          tidy();
+          check(v);
+          if (i + 1 < reals) {
+            v[i + 1] = -m;
+            tidy();
+            check(v);
+          }
+        }
     } else {
       return 2;
     }

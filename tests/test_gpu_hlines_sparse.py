@@ -70,3 +70,19 @@ def test_aligned_second_stage(oracle, M, j):
     for line, bc in ((r2c, "PP"), (mk, "NN"), (np.where(np.arange(2 * M) % 2, -mk, mk), "DD")):
         f = _planes(line, np.array([1.0, -0.5]))
         assert rel_l2(gpu_solve(f, bc + "NNDD", SP), oracle.solve(f, bc + "NNDD", SP)) <= TOL, bc
+
+
+@pytest.mark.parametrize("n", [128, 1024])
+@pytest.mark.parametrize("kind", ["PP", "NN", "DD"])
+def test_one_wave_at_a_quarter(oracle, n, kind):
+    """Sources of one wave whose spectrum is the middle Hermitian item of a line alone (n/4 waves; n/4 or 3n/4 half
+    waves), which the inverse kinds pair with itself."""
+    x = np.arange(n) + 0.5
+    for m in (n // 4, 3 * n // 4):
+        wave = {"PP": np.cos(2 * np.pi * m * (x - 0.5) / n + 0.3), "NN": np.cos(np.pi * m * x / n),
+                "DD": np.sin(np.pi * m * x / n)}[kind]
+        for bc, f in ((kind + "NNDD", _planes(wave, np.array([1.0, -0.5]))),
+                      ("NN" + kind + "DD", _planes(wave, np.array([1.0, -0.5, 0.25, 2.0])).transpose(0, 2, 1)),
+                      ("PP" + kind + "DD", _planes(wave, np.array([1.0, -0.5, 0.25, 2.0])).transpose(0, 2, 1))):
+            f = np.ascontiguousarray(f)
+            assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, (bc, m)
