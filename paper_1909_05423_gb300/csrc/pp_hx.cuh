@@ -180,9 +180,11 @@ __device__ __forceinline__ double hx_to_double(hx v, int E) {
 }
 
 // Scale of a line from its largest magnitude and its sum of magnitudes: the largest power of two with
-// S <= max(am_e / mx, as_e / l1) for every bound e.
+// S <= max(am_e / mx, as_e / l1) for every bound e.  l1 is summed in units of 2^12, so that the up to 2052 magnitudes
+// of a line stay within FP32's range; it is infinite or NaN for non-finite values only.
+constexpr float kHxSum = 0x1p-12f;
 struct HScale {
-  float am[6], as[6];  // limit / (bound per unit of the largest magnitude, of the sum)
+  float am[6], as[6];  // limit / (bound per unit of the largest magnitude, of the sum in units of 2^12)
   int n;
   int out;             // exponent of the scale that the products took off
 };
@@ -193,7 +195,7 @@ inline HScale hx_bounds(bool iv, bool inv, bool c2c, const int* rad, int nst) {
   HScale b = {};
   auto add = [&](double per_max, double per_sum) {
     b.am[b.n] = (float)(0.95 * 0x1p31 / per_max);
-    b.as[b.n] = (float)(0.95 * 0x1p31 / per_sum);
+    b.as[b.n] = (float)(0.95 * 0x1p31 * kHxSum / per_sum);
     b.n++;
   };
   // before the first stage: the values themselves (type IV), sums of two pairs (inverse kinds)
@@ -221,7 +223,7 @@ inline HScale hx_bounds(bool iv, bool inv, bool c2c, const int* rad, int nst) {
 }
 __device__ __forceinline__ void hx_stat(float& mx, float& l1, float v) {
   mx = fmaxf(mx, fabsf(v));
-  l1 += fabsf(v);
+  l1 = __fmaf_rn(fabsf(v), kHxSum, l1);
 }
 __device__ __forceinline__ float hx_scale(const HScale& b, float mx, float l1) {
   const float rm = __frcp_rn(mx), rl = __frcp_rn(l1);

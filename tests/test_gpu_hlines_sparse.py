@@ -86,3 +86,11 @@ def test_one_wave_at_a_quarter(oracle, n, kind):
                       ("PP" + kind + "DD", _planes(wave, np.array([1.0, -0.5, 0.25, 2.0])).transpose(0, 2, 1))):
             f = np.ascontiguousarray(f)
             assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, (bc, m)
+
+
+@pytest.mark.parametrize("bc", ["NNDDDD", "PPPPDD", "DNNDDD"])
+def test_large_magnitudes(oracle, bc):
+    """Lines whose sum of magnitudes is beyond FP32's range while the transforms stay within it."""
+    f = np.random.default_rng(84).uniform(-5e35, 5e35, (4, 4, 2048))
+    for g in (f, np.ascontiguousarray(f.transpose(0, 2, 1))):
+        assert rel_l2(gpu_solve(g, bc, SP), oracle.solve(g, bc, SP)) <= TOL

@@ -29,7 +29,8 @@ def exe(tmp_path_factory):
 
 # random: dense lines.  fours, few: lines of a few cells, whose scale the sum of magnitudes sets.  aligned: lines whose
 # cells add up in one of the values that the butterflies take re + im or re - im of.  modes: one or two coefficients.
-@pytest.mark.parametrize("family", ["random", "fours", "few", "aligned", "modes"])
+# huge: magnitudes whose sum is beyond FP32's range while every result is within it.
+@pytest.mark.parametrize("family", ["random", "fours", "few", "aligned", "modes", "huge"])
 def test_lines(exe, family):
     with cf.ThreadPoolExecutor(5) as ex:
         runs = list(ex.map(lambda M: subprocess.run([exe, family, str(M)], capture_output=True, text=True, timeout=300),
