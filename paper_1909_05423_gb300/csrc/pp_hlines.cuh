@@ -42,31 +42,33 @@ __device__ __forceinline__ htwb hld(const htwb* p) {
   return htwb{v.x, v.y};
 }
 
-// Streamed inputs bypass L1, which then keeps the twiddle tables (28 KB beside three CTAs' shared memory).
+// Streamed inputs bypass L1, which then keeps the twiddle tables (28 KB beside three CTAs' shared memory).  They are
+// the kernel before's output, or (z lines) this kernel's own: coherent loads, volatile and with a memory clobber so
+// that the compiler keeps them behind pdl_wait().
 __device__ __forceinline__ df hld1(const double* p) {
   double a;
-  asm("ld.global.nc.L1::no_allocate.f64 %0, [%1];\n" : "=d"(a) : "l"(__cvta_generic_to_global(p)));
+  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];\n" : "=d"(a) : "l"(__cvta_generic_to_global(p)) : "memory");
   return df_from_double(a);
 }
 __device__ __forceinline__ df hld1(const float2* p) {
   float a, b;
-  asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];\n" : "=f"(a), "=f"(b) : "l"(__cvta_generic_to_global(p)));
+  asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];\n" : "=f"(a), "=f"(b) : "l"(__cvta_generic_to_global(p)) : "memory");
   return df{a, b};
 }
 __device__ __forceinline__ void hld2(const double* p, df* t) {
   double a, b;
-  asm("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];\n" : "=d"(a), "=d"(b) : "l"(__cvta_generic_to_global(p)));
+  asm volatile("ld.global.L1::no_allocate.v2.f64 {%0, %1}, [%2];\n" : "=d"(a), "=d"(b) : "l"(__cvta_generic_to_global(p)) : "memory");
   t[0] = df_from_double(a);
   t[1] = df_from_double(b);
 }
 __device__ __forceinline__ void hld2(const float2* p, df* t) {
-  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];\n"
-      : "=f"(t[0].hi), "=f"(t[0].lo), "=f"(t[1].hi), "=f"(t[1].lo) : "l"(__cvta_generic_to_global(p)));
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+      : "=f"(t[0].hi), "=f"(t[0].lo), "=f"(t[1].hi), "=f"(t[1].lo) : "l"(__cvta_generic_to_global(p)) : "memory");
 }
 // four adjacent reals of an x line (32-byte aligned FP64, or spill pairs)
 __device__ __forceinline__ void hld4(const double* p, df* t) {
   double a, b, c, d;
-  asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];\n" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(__cvta_generic_to_global(p)));
+  asm volatile("ld.global.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];\n" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(__cvta_generic_to_global(p)) : "memory");
   t[0] = df_from_double(a);
   t[1] = df_from_double(b);
   t[2] = df_from_double(c);

@@ -110,12 +110,12 @@ __device__ __forceinline__ void for_items(const LineArgs& a, int nl, const FastD
 // Vector access to 2 or 4 consecutive reals at a real offset that is a multiple of 2 / 4
 // (rows of x tiles are 16-byte aligned; the host checks the array pointers).
 // raw(): the loaded bits, cvt(): their conversion to R (split so that a batch of loads can be
-// issued before the first conversion waits for its data).
+// issued before the first conversion waits for its data).  Plain loads, as in Io (pp_arith.cuh).
 template <class R, class S> struct Vec;
 template <> struct Vec<df, double> {
   using raw_t = double2;
   __device__ static __forceinline__ raw_t raw(const double* p, long long o) {
-    return __ldg(reinterpret_cast<const double2*>(p + o));
+    return *reinterpret_cast<const double2*>(p + o);
   }
   __device__ static __forceinline__ void cvt(raw_t a, df* v) { v[0] = df_from_double(a.x); v[1] = df_from_double(a.y); }
   __device__ static __forceinline__ void ld2(const double* p, long long o, df* v) { cvt(raw(p, o), v); }
@@ -126,7 +126,7 @@ template <> struct Vec<df, double> {
 template <> struct Vec<df, float2> {
   using raw_t = float4;
   __device__ static __forceinline__ raw_t raw(const float2* p, long long o) {
-    return __ldg(reinterpret_cast<const float4*>(p + o));
+    return *reinterpret_cast<const float4*>(p + o);
   }
   __device__ static __forceinline__ void cvt(raw_t a, df* v) { v[0] = df{a.x, a.y}; v[1] = df{a.z, a.w}; }
   __device__ static __forceinline__ void ld2(const float2* p, long long o, df* v) { cvt(raw(p, o), v); }
@@ -137,7 +137,7 @@ template <> struct Vec<df, float2> {
 template <> struct Vec<float, double> {
   using raw_t = double2;
   __device__ static __forceinline__ raw_t raw(const double* p, long long o) {
-    return __ldg(reinterpret_cast<const double2*>(p + o));
+    return *reinterpret_cast<const double2*>(p + o);
   }
   __device__ static __forceinline__ void cvt(raw_t a, float* v) { v[0] = f32_from_double(a.x); v[1] = f32_from_double(a.y); }
   __device__ static __forceinline__ void ld2(const double* p, long long o, float* v) { cvt(raw(p, o), v); }
@@ -148,7 +148,7 @@ template <> struct Vec<float, double> {
 template <> struct Vec<float, float> {
   using raw_t = float2;
   __device__ static __forceinline__ raw_t raw(const float* p, long long o) {
-    return __ldg(reinterpret_cast<const float2*>(p + o));
+    return *reinterpret_cast<const float2*>(p + o);
   }
   __device__ static __forceinline__ void cvt(raw_t a, float* v) { v[0] = a.x; v[1] = a.y; }
   __device__ static __forceinline__ void ld2(const float* p, long long o, float* v) { cvt(raw(p, o), v); }
@@ -162,7 +162,7 @@ template <class R, class S> struct VecN;
 template <> struct VecN<float, float> {
   static constexpr int V = 4;
   __device__ static __forceinline__ void ld(const float* p, long long o, float* v) {
-    float4 a = __ldg(reinterpret_cast<const float4*>(p + o));
+    float4 a = *reinterpret_cast<const float4*>(p + o);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
   }
   __device__ static __forceinline__ void st(float* p, long long o, const float* v) {
@@ -172,7 +172,7 @@ template <> struct VecN<float, float> {
 template <> struct VecN<df, float2> {
   static constexpr int V = 2;
   __device__ static __forceinline__ void ld(const float2* p, long long o, df* v) {
-    float4 a = __ldg(reinterpret_cast<const float4*>(p + o));
+    float4 a = *reinterpret_cast<const float4*>(p + o);
     v[0] = df{a.x, a.y}; v[1] = df{a.z, a.w};
   }
   __device__ static __forceinline__ void st(float2* p, long long o, const df* v) {
@@ -201,7 +201,7 @@ template <> struct CVec<float, float> {
   static constexpr int VC = 2;
   __device__ static __forceinline__ void ld(const float* p, long long o, int nv, cx<float>* z) {
     if (nv == 2) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(p + o));
+      const float4 v = *reinterpret_cast<const float4*>(p + o);
       z[0] = cx<float>{v.x, v.y};
       z[1] = cx<float>{v.z, v.w};
     } else {
