@@ -84,17 +84,19 @@ typedef struct pp_plan_options {
   int threads_y_inv;
   int cols_y_inv;
   int z_method;    /* periodic z only: 0 = automatic (Sherman-Morrison, or with autotune = 1 the
-                      faster of the two, timed), 1 = Sherman-Morrison, 2 = DFT along z and a
+                      fastest of the Sherman-Morrison sweeps, its partitioned form and the z
+                      transform, timed), 1 = Sherman-Morrison sweeps, 2 = DFT along z and a
                       diagonal solve (needs nz = 2^a 3^b 5^c 7^d <= 4096, else
                       PP_ERR_UNSUPPORTED_SIZE); ignored for non-periodic z */
-  int z_split;     /* non-periodic z only: 0 = automatic (by the grid's size, or with autotune = 1
+  int z_split;     /* 0 = automatic (by the grid's size, or with autotune = 1
                       the fastest of the sweeps and the partitioned solves, timed as a lone launch),
                       1 = Thomas sweeps, 8 / 16 / 32 = partitioned solve: every z line split into
                       chunks of that many rows, one thread per chunk, the chunk carries combined by
                       a short sum or recursive doubling (see pp_plan_z_split).  Needs
                       nz <= 512 x rows (else PP_ERR_UNSUPPORTED_SIZE); other values
-                      PP_ERR_INVALID_ARG; ignored for periodic z, whose Sherman-Morrison solve
-                      always takes the automatic choice */
+                      PP_ERR_INVALID_ARG.  Periodic z: 0 = automatic (the Sherman-Morrison solve on
+                      whole lines or on chunks, by the grid's size or timed, unless z_method is
+                      1 or 2); any of the others = the sweeps */
   int reserved[1]; /* must be zero */
 } pp_plan_options;
 
@@ -251,12 +253,12 @@ size_t pp_plan_device_bytes(const pp_plan* plan);
  * Errors: PP_ERR_INVALID_ARG (NULL). */
 pp_status pp_plan_launch_shapes(const pp_plan* plan, int out[8]);
 
-/* How the plan solves along z: *out = 0 (non-periodic z: Thomas), 1 (periodic z: Sherman-Morrison
- * sweeps) or 2 (periodic z: DFT along z and a diagonal solve), as chosen by options.z_method or the
+/* How the plan solves along z: *out = 0 (non-periodic z: Thomas), 1 (periodic z: Sherman-Morrison)
+ * or 2 (periodic z: DFT along z and a diagonal solve), as chosen by options.z_method or the
  * autotuner.  Errors: PP_ERR_INVALID_ARG (NULL). */
 pp_status pp_plan_z_method(const pp_plan* plan, int* out);
 
-/* The plan's non-periodic z solver: *out = 1 for the Thomas sweeps (one thread per mode runs the
+/* How the plan runs its Thomas or Sherman-Morrison solve: *out = 1 for the sweeps (one thread per mode runs the
  * forward elimination and the back substitution along the whole line), or M = 8, 16 or 32 for the
  * partitioned solve (Sec. "Solution of the Resulting Tridiagonal Matrices", with the sequential
  * sweep replaced as in the parallel alternatives of Sec. "Cyclic Reduction Technique"): each line
@@ -265,8 +267,8 @@ pp_status pp_plan_z_method(const pp_plan* plan, int* out);
  * comes from the chunks nearby (a mode decays along its line) or, for weakly dominant modes, from
  * recursive doubling over ceil(log2(nz / M)) levels.  Same multipliers and results as the sweeps up
  * to rounding; about half again their arithmetic, in exchange for nz / M times the threads.  Chosen
- * by options.z_split, by the grid's size or by the autotuner; periodic z reports 1.  Errors:
- * PP_ERR_INVALID_ARG (NULL). */
+ * by options.z_split, by the grid's size or by the autotuner; a plan that transforms z reports 1.
+ * Errors: PP_ERR_INVALID_ARG (NULL). */
 pp_status pp_plan_z_split(const pp_plan* plan, int* out);
 
 /* ---- Prototype, not used by the solver: a DFT stage on the tensor cores (tcgen05, TMEM). ----

@@ -163,7 +163,8 @@ class Plan:
         return {0: "thomas", 1: "sherman-morrison", 2: "transform"}[v.value]
 
     def z_split(self) -> int:
-        """Rows per chunk of the partitioned z solve (8, 16 or 32), or 1 for the Thomas sweeps."""
+        """Rows per chunk of the partitioned z solve (8, 16 or 32), or 1 for the sweeps (Thomas or
+        Sherman-Morrison) and for plans that transform z."""
         v = ctypes.c_int()
         _lib.check(_lib.load().pp_plan_z_split(self._h, ctypes.byref(v)))
         return v.value

@@ -242,6 +242,7 @@ struct pp_plan {
   // algorithm (zsplit for non-periodic z, zmethod for periodic z); a batched graph may swap these
   // members to the library's shared-GPU settings (pp_solve_batched)
   bool tuned, z_tuned;
+  bool z_auto;          // (autotuned plans) the rows per chunk were the library's to choose
 };
 
 namespace pp {

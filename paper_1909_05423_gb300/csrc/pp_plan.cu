@@ -1119,6 +1119,8 @@ static pp_status autotune(pp_plan* p, bool zmethod_free, bool zsplit_free) {
       if (t < tsm) { tsm = t; sbest = M; }
     }
     p->zsplit = sbest;
+  } else if (p->zfft_ok && zmethod_free) {
+    tsm = time_stage(2);
   }
   // periodic z: those or the z transform, unless the caller chose one
   if (p->zfft_ok && zmethod_free) {
@@ -1249,7 +1251,7 @@ struct SettingsSwap {
       choose_shapes(p, nullptr);
       if (tuned && p->tuned) {
         if (p->z_tuned) {
-          p->zsplit = z_rows_default(p);
+          if (p->z_auto) p->zsplit = z_rows_default(p);
           p->zmethod = ZM_SM;
         }
         continue;
@@ -1443,9 +1445,9 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   const int zreq = opt ? opt->z_method : 0;
   if (zreq == 2 && !zfft_ok)
     return fail(PP_ERR_UNSUPPORTED_SIZE, "z_method 2 (transform) needs periodic z and nz = 2^a 3^b 5^c 7^d <= 4096");
-  // partitioned z solve (non-periodic z; ignored for periodic z): at most 512 chunks per line
-  const int sreq = (opt && !zper) ? opt->z_split : 0;
-  if (sreq > 1) {
+  // partitioned z solve on request (non-periodic z only): at most 512 chunks per line
+  const int sreq = opt ? opt->z_split : 0;
+  if (sreq > 1 && !zper) {
     int G, lgG, P;
     if (!zpart_shape(nz, sreq, dtype == PP_F64 ? 8 : 4, &G, &lgG, &P))
       return fail(PP_ERR_UNSUPPORTED_SIZE, "z_split %d: nz = %d needs more than 512 chunks per line", sreq, nz);
@@ -1479,7 +1481,9 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   p->zfft_ok = zfft_ok;
   if (p->zfft_ok && (s = zfft_tables(p)) != PP_OK) { free_plan(p); return s; }
   p->zmethod = (zreq == 2) ? ZM_FFT : ZM_SM;
-  p->zsplit = sreq ? sreq : z_rows_default(p);
+  // periodic z: the sweeps where the caller chose Sherman-Morrison or gave a split, which is for non-periodic z
+  const bool zauto = sreq == 0 && !(zper && zreq == 1);
+  p->zsplit = zauto ? z_rows_default(p) : zper ? 1 : sreq;
   // Block-scaled line kernels where they exist (powers of two from 64 complex points) and the caller gave no
   // launch shape: 1.3 to 2.2 times as fast as the double-float ones there (pp_hlines.cuh), and closer to FP64.
   if (dtype == PP_F64) {
@@ -1508,10 +1512,11 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   }
   cudaMemset(p->d_status, 0, 4 * sizeof(unsigned));
   if (opt && opt->autotune) {
-    pp_status ts = autotune(p, zreq == 0, sreq == 0);
+    pp_status ts = autotune(p, zreq == 0, zauto);
     if (ts != PP_OK) { free_plan(p); return ts; }
     p->tuned = true;
-    p->z_tuned = zper ? (zreq != 2) : (sreq == 0);
+    p->z_tuned = zper ? (zreq == 0) : zauto;
+    p->z_auto = zauto;
   }
   p->pdl = true;  // (not for the autotuner's concurrent copies)
   *out = p;
@@ -1743,7 +1748,7 @@ pp_status pp_plan_z_method(const pp_plan* p, int* out) {
 
 pp_status pp_plan_z_split(const pp_plan* p, int* out) {
   if (!p || !out) return fail(PP_ERR_INVALID_ARG, "NULL plan or pointer");
-  *out = (p->bc[4] == PP_BC_PERIODIC) ? 1 : p->zsplit;
+  *out = (p->zmethod == ZM_FFT) ? 1 : p->zsplit;
   return PP_OK;
 }
 
