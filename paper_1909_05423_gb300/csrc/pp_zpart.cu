@@ -54,10 +54,18 @@ __device__ __forceinline__ void zp_st(float* p, df v) { *p = df_to_f32(v); }
 __device__ __forceinline__ df zp_f2(float2 v) { return df{v.x, v.y}; }
 __device__ __forceinline__ df zp_f2(const float* v) { return df{v[0], v[1]}; }
 
-// Composition of chunk maps x -> A x + B: (X o Y)(x) = X(Y(x)) = (A_X A_Y) x + (A_X B_Y + B_X).
-__device__ __forceinline__ void zp_compose(df& A, df& B, df Ay, df By) {
-  B = A * By + B;
-  A = A * Ay;
+// Chunk maps x -> A x + B and their composition, (X o Y)(x) = X(Y(x)) = (A_X A_Y) x + (A_X B_Y + B_X).  Where a mode
+// of the CTA runs the near -1 form (N1), A is kept as 1 - A, like the multipliers: a converged chunk has the same A all
+// along the line, and the rounding of an A close to 1, the same in every chunk, would add up to 2^-48 / (1 + w) of
+// the solution (3000 x 48 x 48, source of smooth blobs: relative error 6.2e-14 against 2.6e-14).
+template <bool N1> __device__ __forceinline__ df zp_apply(df A, df B, df x) {
+  if constexpr (N1) return zw_sub<true>(B, A, x);  // (B + x) - (1 - A) x
+  else return A * x + B;
+}
+template <bool N1> __device__ __forceinline__ void zp_compose(df& A, df& B, df Ay, df By) {
+  B = zp_apply<N1>(A, B, By);
+  if constexpr (N1) A = zw_sub<true>(A, A, Ay);    // 1 - A A_y = a + a_y - a a_y
+  else A = A * Ay;
 }
 __device__ __forceinline__ df zp_shfl(df v, int delta, bool up) {
   return up ? df{__shfl_up_sync(0xffffffffu, v.hi, delta), __shfl_up_sync(0xffffffffu, v.lo, delta)}
@@ -70,14 +78,16 @@ constexpr int kZpWindow = 8;
 // Carry of every chunk from the chunk maps of its line.  dir = +1 (forward recurrence): the value
 // that leaves chunk c - 1 (0 for chunk 0); dir = -1 (backward): the one that leaves chunk c + 1 (0 for
 // the last).  sA, sB: one entry per thread.  Every thread of the CTA calls it, with the same `wide`;
-// threads past the line (c >= P) hold the identity map.  `terms`: predecessors that matter to the
-// thread's mode (windowed form).  Contains one barrier.
+// threads past the line (c >= P) hold the zero map: the doubling composes it
+// before the last chunk of a backward line, whose B already holds what enters there.  `terms`: predecessors
+// that matter to the thread's mode (windowed form).  Contains one barrier.
 //
 // Doubling (wide): a warp holds CW = 32 / G consecutive chunks of each of the CTA's G lines (lane =
 // chunk-in-warp x G + line), one segment per line; the segments are scanned with shuffles (log2 CW
 // levels: at level o a chunk composes its map with the one o chunks nearer the start), the segment
 // totals are exchanged through shared memory, and each chunk composes the totals of the segments
-// before its own.
+// before its own.  (A near -1 mode always needs more terms than the window has: N1 comes with `wide`.)
+template <bool N1>
 __device__ __forceinline__ df zp_carry(df A, df B, float2* sA, float2* sB, int c, int P, int col, int G, int lgG,
                                        int dir, bool wide, int terms) {
   const bool fwd = dir > 0;
@@ -93,7 +103,7 @@ __device__ __forceinline__ df zp_carry(df A, df B, float2* sA, float2* sB, int c
       x = zp_f2(sB[t]);
       for (int j = 1; j < nt; j++) {
         t += dir * G;
-        x = zp_f2(sA[t]) * x + zp_f2(sB[t]);
+        x = zp_apply<N1>(zp_f2(sA[t]), zp_f2(sB[t]), x);
       }
     }
     return x;
@@ -106,7 +116,7 @@ __device__ __forceinline__ df zp_carry(df A, df B, float2* sA, float2* sB, int c
   // 1. inclusive scan within the segment
   for (int o = 1; o < cw; o <<= 1) {
     const df An = zp_shfl(A, o * G, fwd), Bn = zp_shfl(B, o * G, fwd);
-    if (fwd ? (ci >= o) : (ci + o < cw)) zp_compose(A, B, An, Bn);
+    if (fwd ? (ci >= o) : (ci + o < cw)) zp_compose<N1>(A, B, An, Bn);
   }
   // the inclusive map of the neighbouring chunk nearer the start (same segment unless at its edge)
   const df An1 = zp_shfl(A, G & 31, fwd), Bn1 = zp_shfl(B, G & 31, fwd);
@@ -121,12 +131,18 @@ __device__ __forceinline__ df zp_carry(df A, df B, float2* sA, float2* sB, int c
   df Lb = df{0.f, 0.f};
   for (int t = 0; t < (fwd ? seg : nseg - 1 - seg); t++) {
     const int j = fwd ? t : nseg - 1 - t;
-    Lb = zp_f2(sA[j * G + col]) * Lb + zp_f2(sB[j * G + col]);
+    Lb = zp_apply<N1>(zp_f2(sA[j * G + col]), zp_f2(sB[j * G + col]), Lb);
   }
   // the carry: the neighbour's output, its segment map applied to L's output (at the segment's
   // edge, L's output itself)
   const bool edge = fwd ? (ci == 0) : (ci == cw - 1);
-  return edge ? Lb : An1 * Lb + Bn1;
+  return edge ? Lb : zp_apply<N1>(An1, Bn1, Lb);
+}
+
+// The near -1 form out of line, as in the sweeps: few CTAs take it, and the others keep their registers.
+__device__ __noinline__ df zp_carry_near1(df A, df B, float2* sA, float2* sB, int c, int P, int col, int G, int lgG,
+                                          int dir) {
+  return zp_carry<true>(A, B, sA, sB, c, P, col, G, lgG, dir, true, 0);
 }
 
 // The multipliers of a line, as stored (pp_zmul.cuh).
@@ -218,11 +234,20 @@ __device__ __forceinline__ void zp_bwd2(df (&v)[M], df u, const ZpRows& R) {
     else fn<S, M, ZP_NEAR>(__VA_ARGS__);                   \
   } while (0)
 
-// x^M for the chunk's map, M a power of two
+// A of a converged chunk, (-w)^M, M a power of two; and 1 - A of one from v = 1 + w, in FP64 (two or three operations
+// a doubling, in the few near -1 CTAs): three double-float roundings of a value that every chunk of the line applies
+// were worth a third of the whole solve's error on 3000 x 48 x 48.
 template <int M> __device__ __forceinline__ df zp_pow(df x) {
 #pragma unroll
   for (int m = 1; m < M; m <<= 1) x = x * x;
   return x;
+}
+template <int M> __device__ __forceinline__ df zp_pow_near1(df v) {
+  double x = (double)v.hi + (double)v.lo;
+#pragma unroll
+  for (int m = 1; m < M; m <<= 1) x = __fma_rn(-x, x, x + x);  // 1 - A^2 = 2 a - a a
+  const float hi = (float)x;
+  return df{hi, (float)(x - (double)hi)};
 }
 
 // CTAs of up to 1024 threads at 64 registers (8 or 16 rows a thread), 512 at 128 (32 rows)
@@ -307,9 +332,10 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
   const df scale = df{a.scale[0], a.scale[1]};
 
   // A of a converged chunk and how many chunks back it reaches
-  df A = zp_pow<M>(n1 ? df{1.f, 0.f} - W.winf : -W.winf);
-  const int terms = A.hi < 0x1p-56f ? 1 : (int)__fdividef(-56.0f, __log2f(fminf(A.hi, 0.999f))) + 1;
-  const bool wide = __any_sync(0xffffffffu, live && terms > kZpWindow);
+  df A = n1 ? zp_pow_near1<M>(W.winf) : zp_pow<M>(-W.winf);
+  const float reach = n1 ? 1.0f - A.hi : A.hi;
+  const int terms = reach < 0x1p-56f ? 1 : (int)__fdividef(-56.0f, __log2f(fminf(reach, 0.999f))) + 1;
+  const bool wide = n1 || __any_sync(0xffffffffu, live && terms > kZpWindow);
   const bool lanes_fast = __all_sync(0xffffffffu, k0 >= W.wlen && k0 + M < n);
   const int var = n1 ? ZP_NEAR : (wide ? ZP_WIDE : (lanes_fast ? ZP_FAST : ZP_TAB));
   ZpRows R;
@@ -336,9 +362,12 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
       }
     // A of a chunk in the prefix (nothing passes through the first chunk, or through the last)
     if (k0 < W.wlen && c > 0 && c < P - 1) {
-      A = df{1.f, 0.f};
+      A = df{n1 ? 0.f : 1.f, 0.f};
 #pragma unroll
-      for (int i = 0; i < M; i++) A = n1 ? zw_neg_mul<true>(A, zp_f2(sW[i])) : zw_neg_mul<false>(A, zp_f2(sW[i]));
+      for (int i = 0; i < M; i++) {
+        const df w = zp_f2(sW[i]);
+        A = n1 ? zw_sub<true>(w, w, A) : zw_neg_mul<false>(A, w);  // N1: 1 - A (1 - v) = v + a - v a
+      }
     }
   }
 
@@ -354,7 +383,8 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
     }
     sQ[tid] = make_float2(y0.hi, y0.lo);
   }
-  df x = zp_carry(A, B, fA, fB, c, P, col, G, lgG, +1, wide, terms);
+  df x = n1 ? zp_carry_near1(A, B, fA, fB, c, P, col, G, lgG, +1)
+            : zp_carry<false>(A, B, fA, fB, c, P, col, G, lgG, +1, wide, terms);
   ZP_DISPATCH(zp_fwd2, v, x, R);
 
   // back substitution; periodic z starts it from c = (y_0 + y_{n-1} / gamma) / (1 + z_0 + z_{n-1} / gamma)
@@ -372,7 +402,8 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
   }
   B = top;
   ZP_DISPATCH(zp_bwd1, v, B, R);
-  x = zp_carry(A, B, bA, bB, c, P, col, G, lgG, -1, wide, terms);
+  x = n1 ? zp_carry_near1(A, B, bA, bB, c, P, col, G, lgG, -1)
+         : zp_carry<false>(A, B, bA, bB, c, P, col, G, lgG, -1, wide, terms);
   if (c == P - 1) x = top;
   ZP_DISPATCH(zp_bwd2, v, x, R);
   if (live) {
