@@ -36,8 +36,7 @@
 // warp is a few contiguous segments) x P chunks.  The singular mode's slots are solved by one more CTA
 // each (pp_zsing.cuh).
 //
-// Arithmetic: double-float (pp_arith.cuh) on the plan's spill type, normalised steps for the
-// double-float spill and unnormalised ones for FP32 (as in the sweeps).  Range report: pp_range.cuh.
+// Arithmetic: double-float (pp_arith.cuh) on the plan's spill type, with the steps of the sweeps.  Range report: pp_range.cuh.
 #include <algorithm>
 #include <atomic>
 
@@ -159,25 +158,21 @@ struct ZpW {
 //  ZP_TAB:  the multipliers come from the thread's rows of sW in shared memory.  (Taken row after row
 //           from the table where they were used, and only by the lanes that needed them, they made the
 //           prefix warps of a CTA three times as slow as the others, which waited at the barriers.)
-//  ZP_WIDE: the same for a CTA whose carries reach further than the window.
 //  ZP_NEAR: the same with the near -1 form of the products (pp_zmul.cuh).
-// Inside the window the first run of a recurrence only feeds carries that enter scaled by A < 2^-7, so
-// it keeps its pairs unnormalised (12 instructions a step instead of 18; their 2^-46 is far below the
-// rounding of the second run).
-enum { ZP_FAST = 0, ZP_TAB = 1, ZP_WIDE = 2, ZP_NEAR = 3 };
+enum { ZP_FAST = 0, ZP_TAB = 1, ZP_NEAR = 2 };
 
-// Steps of the recurrences: unnormalised for the FP32 spill (as in the sweeps, pp_zsolve.cu: zr_fwd,
-// zr_bwd); for the double-float spill the value that goes on is normalised, the difference or product it
-// comes from is not (products and sums read unnormalised pairs: 15 instructions instead of 18).
-template <class S, int V, bool FIRST> __device__ __forceinline__ df zp_step_f(df d, df g, df w) {
-  if constexpr (V != ZP_NEAR && (sizeof(S) == 4 || (V <= ZP_TAB && FIRST))) return mul_u(add_u(d, -g), w);
-  else if constexpr (V == ZP_NEAR) return zw_mul<true>(d - g, w);
-  else return add_u(d, -g) * w;
+// Steps of the recurrences, in both runs those of the sweeps (pp_zsolve.cu: zr_fwd, zr_bwd): normalised for the
+// double-float spill, unnormalised for the FP32 spill.  (Unnormalised first runs and inner steps of the double-float spill
+// took 10 % less time, 256^3 0.109 against 0.125 ms, at about two bits of every carry and step.)
+template <class S, int V> __device__ __forceinline__ df zp_step_f(df d, df g, df w) {
+  if constexpr (V == ZP_NEAR) return zw_mul<true>(d - g, w);
+  else if constexpr (sizeof(S) == 4) return mul_u(add_u(d, -g), w);
+  else return (d - g) * w;
 }
-template <class S, int V, bool FIRST> __device__ __forceinline__ df zp_step_b(df g, df w, df u) {
-  if constexpr (V != ZP_NEAR && (sizeof(S) == 4 || (V <= ZP_TAB && FIRST))) return add_u(g, -mul_u(w, u));
-  else if constexpr (V == ZP_NEAR) return zw_sub<true>(g, w, u);
-  else return g - mul_u(w, u);
+template <class S, int V> __device__ __forceinline__ df zp_step_b(df g, df w, df u) {
+  if constexpr (V == ZP_NEAR) return zw_sub<true>(g, w, u);
+  else if constexpr (sizeof(S) == 4) return add_u(g, -mul_u(w, u));
+  else return g - w * u;
 }
 
 struct ZpRows {
@@ -197,7 +192,7 @@ __device__ __forceinline__ void zp_fwd1(df (&v)[M], df& B, const ZpRows& R, df s
   for (int i = 0; i < M; i++) {
     v[i] = (sizeof(S) == 4) ? mul_u(v[i], scale) : v[i] * scale;
     track(dmax, v[i].hi);
-    B = zp_step_f<S, V, true>(v[i], B, R.mult<V>(i));
+    B = zp_step_f<S, V>(v[i], B, R.mult<V>(i));
   }
 }
 // g_k from the true carry, in place of d_k; rounded for the FP32 spill as the sweeps round it between
@@ -206,7 +201,7 @@ template <class S, int M, int V>
 __device__ __forceinline__ void zp_fwd2(df (&v)[M], df& g, const ZpRows& R) {
 #pragma unroll
   for (int i = 0; i < M; i++) {
-    g = zp_step_f<S, V, false>(v[i], g, R.mult<V>(i));
+    g = zp_step_f<S, V>(v[i], g, R.mult<V>(i));
     v[i] = (sizeof(S) == 4) ? df{df_to_f32(g), 0.0f} : g;
   }
 }
@@ -214,14 +209,14 @@ __device__ __forceinline__ void zp_fwd2(df (&v)[M], df& g, const ZpRows& R) {
 template <class S, int M, int V>
 __device__ __forceinline__ void zp_bwd1(const df (&v)[M], df& u, const ZpRows& R) {
 #pragma unroll
-  for (int i = M - 1; i >= 0; i--) u = zp_step_b<S, V, true>(v[i], R.mult<V>(i), u);
+  for (int i = M - 1; i >= 0; i--) u = zp_step_b<S, V>(v[i], R.mult<V>(i), u);
 }
 // ... and from the true carry, keeping the values
 template <class S, int M, int V>
 __device__ __forceinline__ void zp_bwd2(df (&v)[M], df u, const ZpRows& R) {
 #pragma unroll
   for (int i = M - 1; i >= 0; i--) {
-    u = zp_step_b<S, V, false>(v[i], R.mult<V>(i), u);
+    u = zp_step_b<S, V>(v[i], R.mult<V>(i), u);
     v[i] = u;
   }
 }
@@ -230,7 +225,6 @@ __device__ __forceinline__ void zp_bwd2(df (&v)[M], df u, const ZpRows& R) {
   do {                                                     \
     if (var == ZP_FAST) fn<S, M, ZP_FAST>(__VA_ARGS__);    \
     else if (var == ZP_TAB) fn<S, M, ZP_TAB>(__VA_ARGS__); \
-    else if (var == ZP_WIDE) fn<S, M, ZP_WIDE>(__VA_ARGS__); \
     else fn<S, M, ZP_NEAR>(__VA_ARGS__);                   \
   } while (0)
 
@@ -337,7 +331,7 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
   const int terms = reach < 0x1p-56f ? 1 : (int)__fdividef(-56.0f, __log2f(fminf(reach, 0.999f))) + 1;
   const bool wide = n1 || __any_sync(0xffffffffu, live && terms > kZpWindow);
   const bool lanes_fast = __all_sync(0xffffffffu, k0 >= W.wlen && k0 + M < n);
-  const int var = n1 ? ZP_NEAR : (wide ? ZP_WIDE : (lanes_fast ? ZP_FAST : ZP_TAB));
+  const int var = n1 ? ZP_NEAR : (lanes_fast ? ZP_FAST : ZP_TAB);
   ZpRows R;
   R.winf = W.winf;
   R.w = sW;
