@@ -887,36 +887,49 @@ static pp_status run_stage(pp_plan* p, int stage, const void* f, void* u, int tr
   return PP_OK;
 }
 
-// Rows per chunk of the z solve when nobody chose them (1: the sweeps), by what was measured (GB300, z
-// stage alone; sweeps / 8 rows / 16 rows, ms):
-//   FP64   32^3 0.028/0.011/0.013   128^3 0.122/0.022/0.026   256^3 0.309/0.113/0.104
-//          256 x 384^2 0.379/0.248/0.225   256 x 512^2 0.471/0.432/0.387   1024 x 512^2 1.63/2.05/1.64
-//          1024^3 4.32/8.2/6.5   4095 x 64^2 3.37/0.197/0.180
-//          periodic z: 192^3 0.246/0.076/0.082   512^3 1.162/1.126/1.163
-//   mixed  256 x 320^2 0.240/0.156/0.137   256 x 448^2 0.299/0.301/0.262   64 x 512^2 0.092/0.113/0.105
-//          512^3 0.61/0.83/0.67   periodic z: 256^3 0.274/0.133/0.145
-// and on longer lines (sweeps / 16 rows):
-//   FP64   300 x 448 x 512 0.477/0.435   600 x 448 x 512 0.914/0.917   800 x 256 x 448 0.948/0.635
-//          1138 x 224 x 448 1.214/1.040   1138 x 288 x 512 1.425/1.534   1138 x 448 x 512 1.571/2.387
-//   mixed  300 x 384^2 0.296/0.253   300 x 448 x 512 0.375/0.388   420 x 320 x 512 0.419/0.394
-//          600 x 384^2 0.534/0.629   1138 x 160 x 512 0.700/0.741   1138 x 288 x 512 0.981/1.350
-//          periodic z, 8 rows: 1138 x 288 x 512 1.49/2.37
-// The sweeps read and write at the copy bandwidth once their threads (one per real slot) fill the GPU;
-// below that a line's serial chain sets their time, whatever the number of lines.  The partitioned solve
-// does 1.5 times their arithmetic and takes 6 ps a value, up to 9 where a CTA of long lines leaves
-// much of an SM's threads idle.  So the number of slots at which the two cross falls with the rows, and
-// is lower for the FP32 spill, whose sweeps move less; the steps below stay under it.  16 rows a chunk do
-// less carry work, 8 give twice the threads: worth it up to 8 M values, and for periodic z, whose q terms
-// weigh on the first chunks.
+// Rows per chunk of the z solve when nobody chose them (1: the sweeps).
+// The sweeps read and write at the copy bandwidth once their threads (one per real slot) fill the GPU; below that
+// a line's serial chain sets their time, whatever the number of lines.  The partitioned solve does 1.5 times
+// their arithmetic and takes 7 ps a value, up to 9 where a CTA of long lines leaves much of an SM's threads idle, and
+// on lines of a few rows its CTAs are a warp or two each and cost more than the sweeps take in all.  So the
+// number of slots (lines) up to which it is the faster one rises with the rows, stays, and falls again; it is lower
+// for the FP32 spill, whose sweeps move less.  The steps below stay under what was measured (GB300).
+// Whole solves, us, sweeps / 8 rows:
+//   FP64      8 rows     4 k 50.9/51.9    16 k 67.4/69.8   128 k 77.6/97.7    256 k 124/147
+//            16 rows     4 k 56.2/51.6    16 k 72.0/72.1    36 k 63.5/76.6
+//            24 rows    16 k 80.1/72.6    36 k 73.7/77.4    96 k 118/118
+//            32 rows    36 k 90.6/81.7   128 k 203/197     192 k 305/309
+//            48 rows   128 k 271/255     192 k 423/416     224 k 577/577
+//           128 rows   128 k 624/547     224 k 1350/1328   256 k 1066/1055
+//   periodic 16 rows     4 k 60.1/54.1    36 k 66.6/79.3    24 rows 64 k 109/101   128 k 204/205
+//            32 rows    64 k 147/115     256 k 382/363     128 rows 192 k 1044/1015   256 k 1114/1144
+//   mixed     8 rows    16 k 33.8/30.0    64 k 37.8/54.7    24 rows 16 k 41.9/42.6   64 k 57.6/65.7
+//            32 rows    64 k 67.1/67.3   128 k 106/104     192 k 142/155
+//            64 rows   128 k 189/174     192 k 259/263     128 rows 192 k 475/473   224 k 617/624
+//   periodic  8 rows    16 k 31.5/32.5    16 rows 16 k 39.7/38.0   36 k 43.8/51.1
+//            24 rows    96 k 87.2/85.7    32 rows 64 k 76.1/75.2  224 k 243/220    128 rows 224 k 708/692
+// z stage alone, ms, sweeps / 16 rows:
+//   FP64  256 x 448 x 512 0.426/0.404   256 x 512^2 0.451/0.461   300 x 448 x 512 0.494/0.504   301 x 384 x 512 0.436/0.430
+//         440 x 320 x 512 0.616/0.508   600 x 384 x 512 0.836/0.889   600 x 256 x 512 0.778/0.592   800 x 192 x 448 0.890/0.526
+//         1138 x 160 x 512 1.009/0.909   1138 x 288 x 512 1.43/1.53   4095 x 64^2 3.37/0.201   1024^3 4.3/6.5
+//         periodic (8 rows): 512^3 1.130/1.254   600 x 256 x 384 0.973/0.770   1000 x 256 x 384 1.51/1.01
+//   mixed 256 x 384 x 512 0.283/0.264   300 x 448 x 512 0.375/0.388   420 x 320 x 512 0.419/0.394   600 x 384^2 0.534/0.629
+//         1138 x 160 x 512 0.700/0.741   512^3 0.61/0.67   periodic (8 rows): 256 x 448 x 512 0.479/0.475   1138 x 288 x 512 1.49/2.37
+// 16 rows a chunk do less carry work, 8 give twice the threads: worth it up to 128 rows a line or 8 M values
+// (128 x 512^2 0.229 / 0.244 ms, 3000 x 48^2 0.092 / 0.076), and for periodic z, whose q terms weigh on the first
+// chunks.
 static int z_rows_default(const pp_plan* p) {
   const bool zper = p->bc[4] == PP_BC_PERIODIC;
-  const bool f64 = p->dtype == PP_F64;
-  long long most;  // slots
-  if (zper) most = p->nz > 512 ? 110000 : f64 ? 290000 : 230000;
-  else if (f64) most = p->nz <= 300 ? 290000 : p->nz <= 600 ? 200000 : 90000;
-  else most = p->nz <= 300 ? 200000 : p->nz <= 450 ? 160000 : 60000;
-  if (p->splane > most) return 1;
-  int M = (zper || p->splane * p->nz <= (8LL << 20)) ? 8 : 16;
+  struct Step { int rows; int slots; };  // lines of up to `rows` rows: the partitioned solve up to `slots` slots
+  static const Step steps[2][2][9] = {
+      {{{24, 16500}, {32, 100000}, {100, 140000}, {300, 197000}, {450, 160000}, {1 << 20, 60000}},
+       {{10, 0}, {16, 20000}, {24, 30000}, {512, 230000}, {1 << 20, 110000}}},
+      {{{10, 2048}, {16, 8192}, {24, 20000}, {32, 110000}, {64, 190000}, {256, 230000}, {300, 200000}, {600, 170000}, {1 << 20, 90000}},
+       {{10, 0}, {16, 8192}, {24, 100000}, {64, 260000}, {512, 200000}, {1 << 20, 110000}}}};
+  const Step* t = steps[p->dtype == PP_F64][zper];
+  while (p->nz > t->rows) t++;
+  if (p->splane > t->slots) return 1;
+  int M = (zper || p->nz <= 128 || p->splane * p->nz <= (8LL << 20)) ? 8 : 16;
   int G, lgG, P;
   for (; M <= 32; M *= 2)
     if (zpart_shape(p->nz, M, (int)p->elem, &G, &lgG, &P)) return M;

@@ -55,3 +55,16 @@ def test_reported_split():
     plan = pp.Plan((64, 8, 12), "NNDDPP", sp, options={"z_split": 8, "autotune": 1})
     assert plan.z_split() == 1 and plan.z_method() in ("sherman-morrison", "transform")
     plan.close()
+
+
+@pytest.mark.parametrize("shape,bc,dtype,want", [
+    ((8, 512, 512), "NNDDNN", "f64", 1), ((2, 256, 256), "PPDDDD", "f64", 1), ((32, 512, 512), "NNDDNN", "f64", 1),
+    ((8, 256, 512), "NNDDNN", "mixed_f64io", 1), ((3, 448, 448), "NNDDPP", "f64", 1), ((12, 256, 256), "NNDDPP", "mixed_f64io", 1),
+    ((32, 256, 256), "NNDDNN", "f64", 8), ((256, 256, 256), "NNDDNN", "f64", 16), ((64, 64, 64), "NNDDNN", "mixed_f64io", 8),
+    ((192, 192, 192), "NNDDPP", "f64", 8)])
+def test_default_by_size(shape, bc, dtype, want):
+    """Short lines of large planes take the sweeps, which are done with them in less time than the chunks' CTAs need."""
+    import paper_1909_05423_gb300 as pp
+    plan = pp.Plan(shape, bc, (0.1, 0.1, 0.1), dtype)
+    assert plan.z_split() == want
+    plan.close()
