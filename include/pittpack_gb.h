@@ -184,6 +184,10 @@ pp_status pp_fold_bc(pp_plan* plan, const void* f_in, void* f_out, const void* c
  * up to 32 concurrent graph branches (measured: 8 -> 32 took 64 uneven grids from 4.19 to 4.04 ms
  * FP64, 2.26 to 2.13 ms FP32); members that share a plan share its workspace and run
  * one after another on one branch.
+ * In a graph the FP64-class lines of fewer than 256 complex points (x or y lines of fewer than 512 cells,
+ * complex columns of fewer than 256) take the double-float kernels, which are the faster ones where the branches share
+ * the GPU; pp_solve takes the block-scaled ones (see threads_x).  So a member's result may differ from
+ * pp_solve's by rounding, within the accuracy of either (~1e-14 a transform).
  * Autotuned members (options.autotune = 1) carry the settings that were fastest for each plan
  * alone, which in a shared graph can lose to the default ones (measured: 64 uneven grids, 5.36
  * against 4.30 ms FP64).  So the first call over a list of plans that includes autotuned members

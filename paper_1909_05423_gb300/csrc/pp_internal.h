@@ -239,8 +239,8 @@ struct pp_plan {
   // 1 = Thomas (Sherman-Morrison) sweeps, M = partitioned solve with M rows per chunk
   int zsplit;
   // created with autotune = 1 (launch shapes timed), and whether the autotuner also chose the z
-  // algorithm (zsplit for non-periodic z, zmethod for periodic z); a batched graph may swap these
-  // members to the library's shared-GPU settings (pp_solve_batched)
+  // algorithm (zsplit for non-periodic z, zmethod for periodic z); a batched graph may run
+  // these members with the library's shared-GPU settings (pp_solve_batched)
   bool tuned, z_tuned;
   bool z_auto;          // (autotuned plans) the rows per chunk were the library's to choose
 };

@@ -19,9 +19,12 @@
 #include <cstdlib>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "pp_internal.h"
@@ -1206,80 +1209,53 @@ void evict_plan(const pp_plan* p) {
 }
 }  // namespace
 
-// Launch settings of a plan that a batched graph may swap: launch shapes and the z algorithm.
-struct PlanSettings {
-  int threads_x[2], lpc_x[2], ldm_x, threads_y[2], lpc_y[2], ldm_y, threads_z, lpc_z, ldm_z, zsplit, zmethod;
-  bool hx_x[2], hx_y[2], pdl;
-};
-static PlanSettings get_settings(const pp_plan* p) {
-  PlanSettings s;
-  for (int d = 0; d < 2; d++) {
-    s.threads_x[d] = p->threads_x[d]; s.lpc_x[d] = p->lpc_x[d];
-    s.threads_y[d] = p->threads_y[d]; s.lpc_y[d] = p->lpc_y[d];
-    s.hx_x[d] = p->hx_x[d]; s.hx_y[d] = p->hx_y[d];
-  }
-  s.ldm_x = p->ldm_x; s.ldm_y = p->ldm_y;
-  s.threads_z = p->threads_z; s.lpc_z = p->lpc_z; s.ldm_z = p->ldm_z;
-  s.zsplit = p->zsplit;
-  s.pdl = p->pdl;
-  s.zmethod = p->zmethod;
-  return s;
-}
-static void set_settings(pp_plan* p, const PlanSettings& s) {
-  for (int d = 0; d < 2; d++) {
-    p->threads_x[d] = s.threads_x[d]; p->lpc_x[d] = s.lpc_x[d];
-    p->threads_y[d] = s.threads_y[d]; p->lpc_y[d] = s.lpc_y[d];
-    p->hx_x[d] = s.hx_x[d]; p->hx_y[d] = s.hx_y[d];
-  }
-  p->ldm_x = s.ldm_x; p->ldm_y = s.ldm_y;
-  p->threads_z = s.threads_z; p->lpc_z = s.lpc_z; p->ldm_z = s.ldm_z;
-  p->zsplit = s.zsplit;
-  p->pdl = s.pdl;
-  p->zmethod = s.zmethod;
-}
-
-// Puts the members of a batch on the library's shared-GPU settings for the scope of one capture, and
-// restores their own afterwards (a captured graph keeps the launch parameters it was captured with).
+// The members of a batch with the library's shared-GPU settings, as copies of the plans for the scope of one
+// capture (a captured graph keeps the launch parameters and the device pointers it was captured with).  The plans
+// themselves are not written: another host thread may be launching a solve of one of them on the same stream.
 //  * Every member: lines of fewer than 256 complex points take the double-float kernels.  The
 //    block-scaled ones hold twice the registers; alone on the GPU they are faster at those lengths (256^3:
 //    0.55 against 0.61 ms), beside 31 other branches their fewer resident warps are not (64 uneven grids:
-//    3.00 against 2.83 ms).
+//    3.00 against 2.83 ms).  And launches do not overlap (launch_pdl).
 //  * Autotuned members, if `tuned` is set: the default launch shapes and, where the autotuner chose the z
 //    algorithm, the default one of its size (the z transform buys a lone plan latency with extra work).
-struct SettingsSwap {
-  std::vector<std::pair<pp_plan*, PlanSettings>> saved;
-  void apply(pp_plan* const* plans, int n, bool tuned) {
+struct BatchMembers {
+  std::vector<std::pair<const pp_plan*, std::unique_ptr<pp_plan>>> copies;
+  std::vector<pp_plan*> members;
+  BatchMembers(pp_plan* const* plans, int n, bool tuned) {
+    static_assert(std::is_trivially_copyable<pp_plan>::value, "a plan is copied by value; the copy owns nothing");
     for (int i = 0; i < n; i++) {
-      pp_plan* p = plans[i];
-      bool seen = false;
-      for (const auto& s : saved) seen |= (s.first == p);
-      if (seen) continue;
-      const PlanSettings own = get_settings(p);
-      saved.emplace_back(p, own);
-      p->pdl = false;
-      for (int d = 0; d < 2; d++) {
-        p->hx_x[d] = own.hx_x[d] && p->fx.M >= 256;
-        p->hx_y[d] = own.hx_y[d] && p->fy.M >= 256;
+      pp_plan* c = nullptr;
+      for (const auto& s : copies)
+        if (s.first == plans[i]) c = s.second.get();
+      if (!c) {
+        copies.emplace_back(plans[i], std::unique_ptr<pp_plan>(new pp_plan(*plans[i])));
+        c = copies.back().second.get();
+        settle(c, *plans[i], tuned);
       }
-      choose_shapes(p, nullptr);
-      if (tuned && p->tuned) {
-        if (p->z_tuned) {
-          if (p->z_auto) p->zsplit = z_rows_default(p);
-          p->zmethod = ZM_SM;
-        }
-        continue;
-      }
-      // the other stages keep the plan's shapes
-      for (int d = 0; d < 2; d++) {
-        if (p->hx_x[d] == own.hx_x[d]) { p->threads_x[d] = own.threads_x[d]; p->lpc_x[d] = own.lpc_x[d]; }
-        if (p->hx_y[d] == own.hx_y[d]) { p->threads_y[d] = own.threads_y[d]; p->lpc_y[d] = own.lpc_y[d]; }
-      }
-      p->threads_z = own.threads_z;
-      p->lpc_z = own.lpc_z;
+      members.push_back(c);
     }
   }
-  ~SettingsSwap() {
-    for (const auto& s : saved) set_settings(s.first, s.second);
+  static void settle(pp_plan* p, const pp_plan& own, bool tuned) {
+    p->pdl = false;
+    for (int d = 0; d < 2; d++) {
+      p->hx_x[d] = own.hx_x[d] && p->fx.M >= 256;
+      p->hx_y[d] = own.hx_y[d] && p->fy.M >= 256;
+    }
+    choose_shapes(p, nullptr);
+    if (tuned && p->tuned) {
+      if (p->z_tuned) {
+        if (p->z_auto) p->zsplit = z_rows_default(p);
+        p->zmethod = ZM_SM;
+      }
+      return;
+    }
+    // the other stages keep the plan's shapes
+    for (int d = 0; d < 2; d++) {
+      if (p->hx_x[d] == own.hx_x[d]) { p->threads_x[d] = own.threads_x[d]; p->lpc_x[d] = own.lpc_x[d]; }
+      if (p->hx_y[d] == own.hx_y[d]) { p->threads_y[d] = own.threads_y[d]; p->lpc_y[d] = own.lpc_y[d]; }
+    }
+    p->threads_z = own.threads_z;
+    p->lpc_z = own.lpc_z;
   }
 };
 
@@ -1366,7 +1342,7 @@ static float time_graph(cudaGraphExec_t g, cudaStream_t st) {
 // extra work.  In a batch graph the members share the GPU and throughput decides, so the first batch
 // over a list of plans with autotuned members times its graph twice on scratch buffers of the
 // members' sizes -- with every member's own settings, and with the shared-GPU settings for the
-// autotuned ones (SettingsSwap) -- and returns which was faster (0 own, 1 shared).  It waits for
+// autotuned ones (BatchMembers) -- and returns which was faster (0 own, 1 shared).  It waits for
 // earlier work on st, which may still use the members' workspaces, and allocates the scratch for
 // the duration of the call; without the memory it keeps the members' own settings.
 static int tune_batch(pp_plan* const* plans, int n, cudaStream_t st) {
@@ -1384,10 +1360,9 @@ static int tune_batch(pp_plan* const* plans, int n, cudaStream_t st) {
   if (ok) {
     float t[2] = {1e30f, 1e30f};
     for (int v = 0; v < 2; v++) {
-      SettingsSwap swap;
-      swap.apply(plans, n, v == 1);
+      const BatchMembers b(plans, n, v == 1);
       cudaGraphExec_t g = nullptr;
-      if (capture_batch(plans, fs.data(), us.data(), n, &g) == PP_OK) {
+      if (capture_batch(b.members.data(), fs.data(), us.data(), n, &g) == PP_OK) {
         t[v] = time_graph(g, st);
         cudaGraphExecDestroy(g);
       }
@@ -1646,9 +1621,8 @@ pp_status pp_solve_batched(pp_plan* const* plans, const void* const* f, void* co
   cudaGraphExec_t exec = nullptr;
   pp_status s;
   {
-    SettingsSwap swap;
-    swap.apply(plans, n, choice == 1);
-    s = capture_batch(plans, f, u, n, &exec);
+    const BatchMembers b(plans, n, choice == 1);
+    s = capture_batch(b.members.data(), f, u, n, &exec);
   }
   if (s != PP_OK) return s;
   cudaError_t e = cudaGraphLaunch(exec, st);
