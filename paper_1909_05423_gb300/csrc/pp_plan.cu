@@ -911,28 +911,35 @@ static pp_status run_stage(pp_plan* p, int stage, const void* f, void* u, int tr
 //            64 rows   128 k 189/174     192 k 259/263     128 rows 192 k 475/473   224 k 617/624
 //   periodic  8 rows    16 k 31.5/32.5    16 rows 16 k 39.7/38.0   36 k 43.8/51.1
 //            24 rows    96 k 87.2/85.7    32 rows 64 k 76.1/75.2  224 k 243/220    128 rows 224 k 708/692
-// z stage alone, ms, sweeps / 16 rows:
-//   FP64  256 x 448 x 512 0.426/0.404   256 x 512^2 0.451/0.461   300 x 448 x 512 0.494/0.504   301 x 384 x 512 0.436/0.430
-//         440 x 320 x 512 0.616/0.508   600 x 384 x 512 0.836/0.889   600 x 256 x 512 0.778/0.592   800 x 192 x 448 0.890/0.526
-//         1138 x 160 x 512 1.009/0.909   1138 x 288 x 512 1.43/1.53   4095 x 64^2 3.37/0.201   1024^3 4.3/6.5
-//         periodic (8 rows): 512^3 1.130/1.254   600 x 256 x 384 0.973/0.770   1000 x 256 x 384 1.51/1.01
-//   mixed 256 x 384 x 512 0.283/0.264   300 x 448 x 512 0.375/0.388   420 x 320 x 512 0.419/0.394   600 x 384^2 0.534/0.629
-//         1138 x 160 x 512 0.700/0.741   512^3 0.61/0.67   periodic (8 rows): 256 x 448 x 512 0.479/0.475   1138 x 288 x 512 1.49/2.37
-// 16 rows a chunk do less carry work, 8 give twice the threads: worth it up to 128 rows a line or 8 M values
-// (128 x 512^2 0.229 / 0.244 ms, 3000 x 48^2 0.092 / 0.076), and for periodic z, whose q terms weigh on the first
-// chunks.
+// z stage alone, us, sweeps / the better of 8 and 16 rows:
+//   FP64  100 rows 192 k 172/152    130: 175 k 203/182    161: 163 k 242/221  175 k 238/254    200: 163 k 303/254
+//         256: 175 k 358/320  229 k 426/403  262 k 451/459    300: 192 k 473/424  229 k 494/504   420: 175 k 551/559  192 k 614/584
+//         600: 163 k 828/736  175 k 748/815  197 k 836/889    800: 86 k 890/526    1138: 82 k 1009/909  147 k 1425/1534
+//         4095: 4 k 3370/201    1024: 1 M 4300/6500
+//   mixed 100 rows 147 k 106/102    161: 147 k 162/156  163 k 162/174    200: 163 k 217/205  175 k 207/231    256: 192 k 289/260
+//         300: 163 k 309/283  175 k 291/313    420: 163 k 418/406    600: 114 k 539/510  131 k 530/580    1138: 82 k 700/741
+//   periodic FP64  100: 204 k 231/213    161: 204 k 395/383    200: 192 k 418/416  204 k 397/440    256: 229 k 551/540  300: 204 k 637/625
+//         229 k 684/700    420: 163 k 812/727  175 k 743/791    512: 163 k 955/794  262 k 1130/1254    1000: 98 k 1506/1014
+//   periodic mixed  100: 229 k 225/209    161: 163 k 322/280  175 k 285/311    200: 163 k 328/315  192 k 371/369    256: 229 k 489/475
+//         300: 114 k 432/407  131 k 446/463  229 k 576/805 (CTAs of 608 threads: one an SM)    512: 163 k 782/696  229 k 889/981
+// 16 rows a chunk do less carry work, 8 give twice the threads: worth it up to 160 rows a line (130 rows 182 / 213) or 8 M
+// values, and for periodic z, whose q terms weigh on the first chunks.
 static int z_rows_default(const pp_plan* p) {
   const bool zper = p->bc[4] == PP_BC_PERIODIC;
   struct Step { int rows; int slots; };  // lines of up to `rows` rows: the partitioned solve up to `slots` slots
-  static const Step steps[2][2][9] = {
-      {{{24, 16500}, {32, 100000}, {100, 140000}, {300, 197000}, {450, 160000}, {1 << 20, 60000}},
-       {{10, 0}, {16, 20000}, {24, 30000}, {512, 230000}, {1 << 20, 110000}}},
-      {{{10, 2048}, {16, 8192}, {24, 20000}, {32, 110000}, {64, 190000}, {256, 230000}, {300, 200000}, {600, 170000}, {1 << 20, 90000}},
-       {{10, 0}, {16, 8192}, {24, 100000}, {64, 260000}, {512, 200000}, {1 << 20, 110000}}}};
+  constexpr int kMaxRows = 1 << 20;
+  static const Step mixed[] = {{10, 256}, {24, 16500}, {32, 100000}, {100, 140000}, {240, 147000}, {280, 197000}, {450, 160000}, {kMaxRows, 60000}};
+  static const Step mixed_per[] = {{10, 0}, {16, 20000}, {24, 30000}, {110, 230000}, {210, 163000}, {256, 230000}, {400, 115000},
+                                   {512, 160000}, {kMaxRows, 110000}};
+  static const Step f64[] = {{10, 256}, {16, 8192}, {24, 20000}, {32, 110000}, {64, 190000}, {160, 230000}, {240, 165000},
+                             {280, 230000}, {450, 200000}, {600, 165000}, {kMaxRows, 90000}};
+  static const Step f64_per[] = {{10, 0}, {16, 8192}, {24, 100000}, {64, 260000}, {130, 225000}, {240, 190000}, {280, 230000},
+                                 {320, 200000}, {512, 168000}, {kMaxRows, 110000}};
+  static const Step* const steps[2][2] = {{mixed, mixed_per}, {f64, f64_per}};
   const Step* t = steps[p->dtype == PP_F64][zper];
   while (p->nz > t->rows) t++;
   if (p->splane > t->slots) return 1;
-  int M = (zper || p->nz <= 128 || p->splane * p->nz <= (8LL << 20)) ? 8 : 16;
+  int M = (zper || p->nz <= 160 || p->splane * p->nz <= (8LL << 20)) ? 8 : 16;
   int G, lgG, P;
   for (; M <= 32; M *= 2)
     if (zpart_shape(p->nz, M, (int)p->elem, &G, &lgG, &P)) return M;
