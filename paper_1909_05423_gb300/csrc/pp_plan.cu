@@ -593,6 +593,28 @@ static void choose_shapes(pp_plan* p, const pp_plan_options* opt) {
   }
 }
 
+// Whether the block-scaled kernels take lines of M complex points in a grid of `values` cells.  Their CTAs carry twice
+// the values of the double-float ones and a longer chain each, so they lose where a CTA's latency shows: below about
+// one CTA an SM, and along x also in the grids of a few waves whose arrays no longer stay in L2 (their tiles are
+// prefetched by the tile 152 before, which runs at the same time).  Whole solves, us, x lines block-scaled / double-float:
+//   lines of  128: 8192 105/102   32768 294/272   262144 1973/1951   (no size where they win)
+//             256: 16384 275/257   32768 544/534   65536 990/1000   262144 3734/3870
+//             512: 1024 and 2048 within 3 %   8192 284/257   16384 489/478   32768 978/997   131072 4019/4168
+//            1024: 4096 246/224   8192 501/493   16384 870/905   65536 3678/3921
+//            2048: 2048 266/257   4096 458/456   8192 915/952   32768 3677/3865
+// y stage, us, mean of forward and inverse:
+//   256 cells, 1024 columns (2^18 values) 9.2/7.6, 4096 12.9/14.0; 2048 cells, 192 columns 17.8/15.0, 256 17.5/17.9; 1024 cells (512
+//   points, where the double-float kernel takes 16 values a thread) 8 columns 10.5/10.8, 4096 27.6/42
+//   2048 cells and columns of 1024 points: 608 lines are one wave of the double-float kernel (12 us) and half of one here (17)
+//   complex columns of 64 to 512 points: 32 columns of 256 5.0/7.0, 512 of 64 4.4/6.5; of 1024: 64 12.2/10.1, 512 12.9/22
+enum { HXU_X = 0, HXU_Y = 1, HXU_C2C = 2 };
+static bool hx_worth(int M, int use, long long values) {
+  if (!hx_length(M)) return false;
+  if (use == HXU_X) return M > 64 && values >= (M == 128 ? 1LL << 24 : 3LL << 22);
+  if (use == HXU_Y ? M == 512 : M < 1024) return true;
+  return values >= (M == 1024 ? 5LL << 18 : 1LL << 19);
+}
+
 // ------------------------------------------------------------------ line launches
 enum { ST_F64 = 0, ST_F32 = 1, ST_SPILL = 2 };
 
@@ -1479,15 +1501,17 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   // periodic z: the sweeps where the caller chose Sherman-Morrison or gave a split, which is for non-periodic z
   const bool zauto = sreq == 0 && !(zper && zreq == 1);
   p->zsplit = zauto ? z_rows_default(p) : zper ? 1 : sreq;
-  // Block-scaled line kernels where they exist (powers of two from 64 complex points) and the caller gave no
-  // launch shape: 1.3 to 2.2 times as fast as the double-float ones there (pp_hlines.cuh), and closer to FP64.
+  // Block-scaled line kernels where they exist (powers of two from 64 complex points), the caller gave no
+  // launch shape and the grid is large enough: 1.3 to 2.2 times as fast as the double-float ones there
+  // (pp_hlines.cuh), and closer to FP64.
   if (dtype == PP_F64) {
     const bool x0 = !opt || !(opt->threads_x || opt->lines_x), y0 = !opt || !(opt->threads_y || opt->cols_y);
-    p->hx_x[0] = hx_length(p->fx.M) && x0;
+    const long long values = (long long)nx * ny * nz;
+    p->hx_x[0] = x0 && hx_worth(p->fx.M, HXU_X, values);
     p->hx_x[1] = p->hx_x[0] && !(opt && (opt->threads_x_inv || opt->lines_x_inv));
-    p->hx_y[0] = hx_length(p->fy.M) && y0;
+    p->hx_y[0] = y0 && hx_worth(p->fy.M, p->ky == AX_P && p->layout == 0 ? HXU_C2C : HXU_Y, values);
     p->hx_y[1] = p->hx_y[0] && !(opt && (opt->threads_y_inv || opt->cols_y_inv));
-    p->hx_z = p->zfft_ok && hx_length(p->fz.M);
+    p->hx_z = p->zfft_ok && hx_worth(p->fz.M, HXU_C2C, values);
     s = PP_OK;
     if (p->hx_x[0]) s = hx_tables(p->kx, nx, false, p->fx, &p->d_h_x);
     if (s == PP_OK && p->hx_y[0]) s = hx_tables(p->ky, ny, p->layout == 0, p->fy, &p->d_h_y);

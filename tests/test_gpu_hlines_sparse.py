@@ -1,5 +1,6 @@
 """The scale of the block-scaled line kernels on lines of a few cells, whose sum of magnitudes sets it, through whole
-solves against the oracle (1e-12 relative L2, the tolerance of the FP64-class path).  Every plane holds the same line
+solves at 1e-12 relative L2, the tolerance of the FP64-class path: lines along y against the oracle, lines along x,
+which take these kernels in large grids only, against the same solve with the double-float kernels.  Every plane holds the same line
 at another magnitude between 1 and 2: the scale is a power of two, so a line can leave its integers at some
 magnitudes only."""
 import numpy as np
@@ -18,24 +19,45 @@ def _setup(oracle):
     need_gpu()
 
 
-def _planes(line, across):
+def _across(n, values):
+    """Factors of the lines of a plane, so many that the grid has at least `values` cells: the block-scaled kernels
+    are taken from 2^24 cells on along x, from 2^19 on along y."""
+    m = -(-values // (len(MAGS) * n))
+    while m % 2 or any(m % p == 0 for p in range(11, m + 1) if all(p % q for q in range(2, int(p ** 0.5) + 1))):
+        m += 1
+    return np.random.default_rng(n).uniform(-2, 2, max(m, 4))
+
+
+def _x_lines(line):
     """[plane, ny, nx]: MAGS[plane] x line[i] across[j], the line along x."""
+    across = _across(len(line), 1 << 24)
     return np.array(MAGS)[:, None, None] * across[None, :, None] * line[None, None, :]
 
 
-@pytest.mark.parametrize("n", [128, 512, 2048])
+def _y_lines(line):
+    across = _across(len(line), 1 << 19)
+    return np.array(MAGS)[:, None, None] * line[None, :, None] * across[None, None, :]
+
+
+def _check(oracle, f, bc):
+    assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, bc
+
+
+def _check_x(f, bc):
+    assert rel_l2(gpu_solve(f, bc, SP), gpu_solve(f, bc, SP, options=dict(threads_x=128, threads_y=128))) <= TOL, bc
+
+
+@pytest.mark.parametrize("n", [128, 256, 512, 2048])
 @pytest.mark.parametrize("kind", ["DN", "ND"])
 def test_four_cells_type_iv(oracle, n, kind):
     """Cells that meet in one butterfly of the first stage, after the pre-products turned them."""
     for cells in ((5 * n // 8 - 1, 5 * n // 8, 7 * n // 8 - 1, 7 * n // 8), (n // 8 - 1, n // 8, 3 * n // 8 - 1, 3 * n // 8)):
         line = np.zeros(n)
         line[list(cells)] = 1.0
-        f = _planes(line, np.array([1.0, -0.5, 0.25, 2.0]))
-        bc = kind + "NNDD"
-        assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, bc
-        f = np.ascontiguousarray(_planes(line, np.linspace(0.6, 1.7, 6)).transpose(0, 2, 1))
-        bc = "NN" + kind + "DD"
-        assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, bc
+        _check(oracle, _y_lines(line), "NN" + kind + "DD")
+        _check(oracle, _y_lines(line), "PP" + kind + "DD")
+        if n > 128:
+            _check_x(_x_lines(line), kind + "NNDD")
 
 
 def _aligned(M, j):
@@ -58,8 +80,7 @@ def test_aligned_second_stage(oracle, M, j):
     nx = 8
     # complex columns: a real source whose x transform is z in column 1
     f = np.real(z[None, :, None] * np.exp(2j * np.pi * np.arange(nx) / nx)[None, None, :]) * (2.0 / nx)
-    f = np.array(MAGS)[:, None, None] * f
-    assert rel_l2(gpu_solve(f, "PPPPDD", SP), oracle.solve(f, "PPPPDD", SP)) <= TOL
+    _check(oracle, np.array(MAGS)[:, None, None] * f, "PPPPDD")
     # real lines of 2M cells: R2C pairs (u_2k, u_2k+1), the Makhoul order of DCT-II and DST-II
     r2c = np.empty(2 * M)
     r2c[0::2], r2c[1::2] = z.real, z.imag
@@ -67,9 +88,10 @@ def test_aligned_second_stage(oracle, M, j):
     k = np.arange(M // 2)
     mk[4 * k], mk[4 * k + 2] = z[k].real, z[k].imag
     mk[4 * k + 3], mk[4 * k + 1] = z[M - 1 - k].real, z[M - 1 - k].imag
-    for line, bc in ((r2c, "PP"), (mk, "NN"), (np.where(np.arange(2 * M) % 2, -mk, mk), "DD")):
-        f = _planes(line, np.array([1.0, -0.5]))
-        assert rel_l2(gpu_solve(f, bc + "NNDD", SP), oracle.solve(f, bc + "NNDD", SP)) <= TOL, bc
+    for line, kind in ((r2c, "PP"), (mk, "NN"), (np.where(np.arange(2 * M) % 2, -mk, mk), "DD")):
+        _check(oracle, _y_lines(line), "NN" + kind + "DD")
+        if M > 64:
+            _check_x(_x_lines(line), kind + "NNDD")
 
 
 @pytest.mark.parametrize("n", [128, 1024])
@@ -81,16 +103,17 @@ def test_one_wave_at_a_quarter(oracle, n, kind):
     for m in (n // 4, 3 * n // 4):
         wave = {"PP": np.cos(2 * np.pi * m * (x - 0.5) / n + 0.3), "NN": np.cos(np.pi * m * x / n),
                 "DD": np.sin(np.pi * m * x / n)}[kind]
-        for bc, f in ((kind + "NNDD", _planes(wave, np.array([1.0, -0.5]))),
-                      ("NN" + kind + "DD", _planes(wave, np.array([1.0, -0.5, 0.25, 2.0])).transpose(0, 2, 1)),
-                      ("PP" + kind + "DD", _planes(wave, np.array([1.0, -0.5, 0.25, 2.0])).transpose(0, 2, 1))):
-            f = np.ascontiguousarray(f)
-            assert rel_l2(gpu_solve(f, bc, SP), oracle.solve(f, bc, SP)) <= TOL, (bc, m)
+        _check(oracle, _y_lines(wave), "NN" + kind + "DD")
+        _check(oracle, _y_lines(wave), "PP" + kind + "DD")
+        if n > 128:
+            _check_x(_x_lines(wave), kind + "NNDD")
 
 
-@pytest.mark.parametrize("bc", ["NNDDDD", "PPPPDD", "DNNDDD"])
-def test_large_magnitudes(oracle, bc):
+@pytest.mark.parametrize("kind", ["NN", "PP", "DN"])
+def test_large_magnitudes(oracle, kind):
     """Lines whose sum of magnitudes is beyond FP32's range while the transforms stay within it."""
-    f = np.random.default_rng(84).uniform(-5e35, 5e35, (4, 4, 2048))
-    for g in (f, np.ascontiguousarray(f.transpose(0, 2, 1))):
-        assert rel_l2(gpu_solve(g, bc, SP), oracle.solve(g, bc, SP)) <= TOL
+    rng = np.random.default_rng(84)
+    f = np.zeros((6, 1050, 2048))
+    f[:, 5::350] = rng.uniform(-5e35, 5e35, (6, 3, 2048))
+    _check_x(f, kind + "DDDD")
+    _check(oracle, rng.uniform(-5e35, 5e35, (8, 2048, 64)), "DD" + kind + "DD")
