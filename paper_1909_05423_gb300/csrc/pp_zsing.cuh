@@ -15,6 +15,9 @@
 namespace pp {
 
 constexpr int kZsingRows = 16;                          // rows a thread holds
+// Up to here one thread does all rows: six block-wide sums and scans take 24 us however few the rows, one thread 13 us for
+// 8 rows, 17 for 24, 22 for 40 and 25 for 48 (z stage of 16 x 16 lines).
+constexpr int kZsingSerial = 40;
 constexpr size_t kZsingSmem = 64 * sizeof(float2);      // warp totals of a scan
 
 __device__ __forceinline__ df zs_ld(const float2* p) { const float2 v = *p; return df{v.x, v.y}; }
@@ -80,7 +83,7 @@ template <bool REV> __device__ __forceinline__ df block_carry(df A, df B, float2
   return pl == 0 ? x : Ap * x + Bp;
 }
 
-// One thread, any line length (lines of more rows than a CTA holds in registers): the pinned Thomas
+// One thread, any line length (short lines, and lines of more rows than a CTA holds in registers): the pinned Thomas
 // recurrence of rows 1..n-1, whose multipliers -k/(k+1) the table stores as 1 + w.
 template <class S>
 __device__ __noinline__ void zsing_serial(S* base, long long P, int n, df scale, const float2* wt, float& dmax,
@@ -136,7 +139,7 @@ __device__ __noinline__ void zsing_block(const ZArgs& a, int part, float2* sm, f
   const int n = a.nz;
   const df scale = df{a.scale[0], a.scale[1]};
   const int R = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-  if (R > kZsingRows) {
+  if (R > kZsingRows || n <= kZsingSerial) {
     if (threadIdx.x == 0) zsing_serial<S>(base, P, n, scale, a.wtab + a.modes[0].woff, dmax, umax);
     return;
   }

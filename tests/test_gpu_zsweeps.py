@@ -68,3 +68,16 @@ def test_default_by_size(shape, bc, dtype, want):
     plan = pp.Plan(shape, bc, (0.1, 0.1, 0.1), dtype)
     assert plan.z_split() == want
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "mixed_f64io"])
+@pytest.mark.parametrize("nz", [3, 12, 40, 41, 57])
+@pytest.mark.parametrize("bc", ["NNNNNN", "PPNNNN", "PPPPPP"])
+def test_singular_mode_short_lines(oracle, bc, nz, dtype):
+    """The singular mode by one thread (up to 40 rows) and by a CTA, in front of the sweeps and of the chunks."""
+    shape = (nz, 6, 8)
+    sp = (1.0 / 8, 1.0 / 6, 1.0 / nz)
+    f = workloads.uniform_source(shape, seed=97)
+    ref = oracle.solve(f, bc, sp)
+    for options in ({"z_split": 1}, None):
+        assert rel_l2(gpu_solve(f, bc, sp, dtype, options=options), ref) <= TOL[dtype], options
