@@ -21,9 +21,9 @@ namespace pp {
 // z sweeps (pp_zsolve.cu).
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-constexpr unsigned kPdlGrid = 16 * 152;
+constexpr unsigned kPdlCtas = 16;  // CTAs per SM up to which launches overlap
 template <class... P, class... A>
-cudaError_t launch_pdl(bool on, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+cudaError_t launch_pdl(unsigned most, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
                        A... args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -34,7 +34,7 @@ cudaError_t launch_pdl(bool on, void (*kernel)(P...), unsigned grid, unsigned bl
   c.dynamicSmemBytes = smem;
   c.stream = st;
   c.attrs = &attr;
-  c.numAttrs = (on && grid <= kPdlGrid) ? 1 : 0;
+  c.numAttrs = (grid <= most) ? 1 : 0;
   return cudaLaunchKernelEx(&c, kernel, args...);
 }
 
@@ -90,17 +90,16 @@ struct LineArgs {
   const void* haux;
   HScale hs;
   int hdir;
-  int pdl;            // launch_pdl allowed
+  unsigned pdl;       // launch_pdl: CTAs up to which the launch overlaps (0: never)
   int ahead, pf;      // tiles between the one a CTA works on and the one it prefetches into L2; allowed
 };
-// LineArgs::ahead: one tile per SM.  A tile's loads then wait for L2 and not for HBM (ms without / with; two or
+// LineArgs::ahead: the device's SM count, one tile per SM.  A tile's loads then wait for L2 and not for HBM (ms without / with; two or
 // more tiles per SM ahead: less or worse).  x lines: block-scaled 1024^3 5.95 / 5.64 forward, 6.8 / 6.3 back,
 // 512^3 R2C 0.93 / 0.78; FP32 1024^3 2.65 / 2.61 and 2.76 / 2.70, 512^3 R2C 0.444 / 0.355, C2R 0.365 / 0.325.
 // y lines: block-scaled real kinds 6.0 / 5.8; FP32 C2C 0.505 / 0.423.  Block-scaled C2C lines lose 2 % and the
 // FP32 real kinds, which batch their loads, 4 %: they do without (LineArgs::pf).  So do the z lines of the z
 // transform, whose tiles take one sector of every plane: mixed, all-periodic 27.0 / 30.5 for the 1024^3 solve, 3.07 /
 // 2.95 at 512^3, 0.413 / 0.417 at 256^3.
-constexpr int kAhead = 152;
 constexpr int kMaxLpc = 512;  // lines per CTA (bounds the per-line bases in shared memory)
 constexpr int kHostChunks = 8;  // plane chunks of a host-buffer solve (copies overlap transforms)
 
@@ -159,7 +158,7 @@ struct ZArgs {
   unsigned* rstat;
   float dmin;             // 2^-100: below it the double-float low parts are subnormal
   float umax;             // 2^124 / (nx ny): above it the inverse transforms may overflow FP32
-  int pdl;                // launch_pdl allowed
+  unsigned pdl;           // as LineArgs::pdl
   int nsing;              // real slots of the singular mode (0 without one): CTAs at the front of the grid
 };
 // status bits of a plan's device status word
@@ -216,6 +215,7 @@ struct pp_plan {
   // launch shapes
   int threads_x[2], lpc_x[2], ldm_x;  // [0] forward, [1] inverse kernels
   int threads_y[2], lpc_y[2], ldm_y;
+  int sms;              // SMs of the device
   bool pdl;             // overlap the launches of a solve (launch_pdl); batch graphs do not
   // block-scaled line kernels (pp_hlines.cuh): which stages take them ([0] forward, [1] inverse), tables
   bool hx_x[2], hx_y[2], hx_z;

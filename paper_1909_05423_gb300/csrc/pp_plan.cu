@@ -596,7 +596,7 @@ static void choose_shapes(pp_plan* p, const pp_plan_options* opt) {
 // Whether the block-scaled kernels take lines of M complex points in a grid of `values` cells.  Their CTAs carry twice
 // the values of the double-float ones and a longer chain each, so they lose where a CTA's latency shows: below about
 // one CTA an SM, and along x also in the grids of a few waves whose arrays no longer stay in L2 (their tiles are
-// prefetched by the tile 152 before, which runs at the same time).  Whole solves, us, x lines block-scaled / double-float:
+// prefetched by the tile one per SM before, which runs at the same time).  Whole solves, us, x lines block-scaled / double-float:
 //   lines of  128: 8192 105/102   32768 294/272   262144 1973/1951   (no size where they win)
 //             256: 16384 275/257   32768 544/534   65536 990/1000   262144 3734/3870
 //             512: 1024 and 2048 within 3 %   8192 284/257   16384 489/478   32768 978/997   131072 4019/4168
@@ -620,7 +620,6 @@ enum { ST_F64 = 0, ST_F32 = 1, ST_SPILL = 2 };
 
 // division helpers of one launch
 static void finish_args(LineArgs& a) {
-  a.ahead = kAhead;
   int M = a.fp.M, N = a.N, K;
   // Hermitian-pair kinds handle k and M-k in one item, k <= M/2
   switch (a.kind) {
@@ -670,7 +669,8 @@ cudaError_t launch_lines(const pp_plan* p, int axis, int dir, int io_in, int io_
                          cudaStream_t st, int z0, int nzc) {
   LineArgs a;
   memset(&a, 0, sizeof a);
-  a.pdl = p->pdl;
+  a.ahead = p->sms;
+  a.pdl = p->pdl ? kPdlCtas * (unsigned)p->sms : 0u;
   if (nzc < 0) { z0 = 0; nzc = p->nz; }
   if (z0 < 0 || nzc < 1 || z0 + nzc > p->nz) return cudaErrorInvalidValue;
   const bool dfm = (p->dtype == PP_F64);
@@ -796,7 +796,7 @@ static void zsolve_args(const pp_plan* p, void* data, int transpose, ZArgs& a) {
   split2(p->zscale, a.scale);
   a.transpose = transpose;
   a.nsing = p->singular ? (a.cplx ? 2 : 1) : 0;
-  a.pdl = p->pdl;
+  a.pdl = p->pdl ? kPdlCtas * (unsigned)p->sms : 0u;
   a.rstat = p->d_status;
   a.dmin = 0x1p-100f;
   a.umax = (float)(0x1p124 / ((double)p->nx * (double)p->ny));
@@ -823,6 +823,7 @@ cudaError_t launch_zsolve(const pp_plan* p, void* data, int transpose, cudaStrea
 static cudaError_t launch_zlines(const pp_plan* p, int dir, void* data, cudaStream_t st) {
   LineArgs a;
   memset(&a, 0, sizeof a);
+  a.ahead = p->sms;
   const bool dfm = (p->dtype == PP_F64);
   const long long ncols = p->splane / 2;
   a.N = p->nz;
@@ -844,7 +845,7 @@ static cudaError_t launch_zlines(const pp_plan* p, int dir, void* data, cudaStre
   a.ncols = (int)ncols;
   a.nblk = (int)((ncols + a.tx - 1) / a.tx);
   a.ntiles = a.nblk;
-  a.pf = 0;  // see kAhead
+  a.pf = 0;  // see LineArgs::ahead
   if (p->hx_z) {
     a.fd_gpc = FastDiv::make(1u);
     finish_args(a);
@@ -1076,10 +1077,8 @@ static pp_status autotune(pp_plan* p, bool zmethod_free, bool zsplit_free) {
     const long long tx = std::max(1, p->lpc_y[s0 == 3] / parts);
     return (ncols + tx - 1) / tx * p->nz;
   };
-  int sm_count = 152;
-  cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
   auto time_stage = [&](int s0) -> float {
-    const long long fill = 16LL * sm_count;  // CTAs for several full waves
+    const long long fill = 16LL * p->sms;  // CTAs for several full waves
     int K = 1;
     if (side_ok && s0 != 2) {
       const long long c = std::max(1LL, stage_ctas(s0));
@@ -1477,6 +1476,10 @@ pp_status pp_plan_create(pp_plan** out, int nx, int ny, int nz, const pp_bc bc[6
   for (int i = 0; i < 6; i++) p->bc[i] = bc[i];
   p->dx = dx; p->dy = dy; p->dz = dz;
   p->dtype = dtype;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || p->sms < 1)
+    p->sms = 152;  // (no device: the allocations below report it)
   p->kx = axis_kind(bc[0], bc[1]);
   p->ky = axis_kind(bc[2], bc[3]);
   p->layout = (p->kx == AX_P) ? 0 : (p->ky == AX_P ? 1 : 2);
