@@ -1016,6 +1016,7 @@ namespace {
 struct TuneEnt {
   int dev, nx, ny, nz, dtype, bc[6];
   bool zmethod_free, zsplit_free;  // the z choices below were timed (else the caller's)
+  int hx;                          // line stages that take block-scaled kernels, whose shapes are not timed
   pp_plan_options best;
   int zmethod, zsplit;
 };
@@ -1024,6 +1025,7 @@ std::vector<TuneEnt> g_tune_cache;
 }  // namespace
 
 static pp_status autotune(pp_plan* p, bool zmethod_free, bool zsplit_free) {
+  const int hx = p->hx_x[0] | p->hx_x[1] << 1 | p->hx_y[0] << 2 | p->hx_y[1] << 3;
   int dev = 0;
   cudaGetDevice(&dev);
   {
@@ -1031,7 +1033,7 @@ static pp_status autotune(pp_plan* p, bool zmethod_free, bool zsplit_free) {
     for (const TuneEnt& e : g_tune_cache)
       if (e.dev == dev && e.nx == p->nx && e.ny == p->ny && e.nz == p->nz && e.dtype == p->dtype &&
           memcmp(e.bc, p->bc, sizeof e.bc) == 0 && e.zmethod_free == zmethod_free &&
-          e.zsplit_free == zsplit_free) {
+          e.zsplit_free == zsplit_free && e.hx == hx) {
         choose_shapes(p, &e.best);
         if (zmethod_free) p->zmethod = e.zmethod;
         if (zsplit_free) p->zsplit = e.zsplit;
@@ -1187,6 +1189,7 @@ static pp_status autotune(pp_plan* p, bool zmethod_free, bool zsplit_free) {
   memcpy(ent.bc, p->bc, sizeof ent.bc);
   ent.zmethod_free = zmethod_free;
   ent.zsplit_free = zsplit_free;
+  ent.hx = hx;
   ent.best = best;
   ent.zmethod = p->zmethod;
   ent.zsplit = p->zsplit;
