@@ -134,6 +134,16 @@ def fft_ops(M: int, arith: str) -> float:
     return ops
 
 
+def _block_scaled(axis: str, N: int, points: int) -> bool:
+    """Whether a default FP64-class plan takes the block-scaled kernels for real lines of N cells (the rule of
+    hx_worth in csrc/pp_plan.cu)."""
+    if N & (N - 1) or not 128 <= N <= 2048:
+        return False
+    if axis == "x":
+        return N > 128 and points >= (2 ** 24 if N == 256 else 3 * 2 ** 22)
+    return N == 1024 or points >= (5 * 2 ** 18 if N == 2048 else 2 ** 19)
+
+
 def line_ops_per_real(kind: str, N: int, arith: str) -> float:
     """Lane instructions per real point of one real line transform of length N (complex FFT of N/2
     points plus the pre/post-processing of the kind): DCT-II/DST-II (Hermitian-pair split and
@@ -660,7 +670,7 @@ def run_ours(args):
         d["hbm_frac"] = d["hbm_gbs"] / peak
         if name in kinds:
             N = nx_ if name[0] == "x" else ny_
-            d["arith"] = "hx" if N & (N - 1) == 0 and 128 <= N <= 2048 else "df"
+            d["arith"] = "hx" if _block_scaled(name[0], N, npts) else "df"
             opr = line_ops_per_real(kinds[name], N, d["arith"])
             d["fp32_ops_per_point"] = opr
             d["alu_tops"] = opr * npts / (per[k] * 1e-3) / 1e12
@@ -750,7 +760,8 @@ def run_ours(args):
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_all, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "f64 I/O, double-float (2xf32) transforms and z-solve",
+            "vs_baseline": None,
+            "dtype": "f64 I/O, block-scaled (int32 + f32) or double-float (2xf32) transforms, double-float z-solve",
             "data": "synthetic (seeded U[-1,1], mean removed; generated on device)",
             "config": {"workload": "%s FP64 Neumann-x/Dirichlet-y/Neumann-z, U[-1,1] source" %
                                    ("%d^3" % n if not args.shape else "%dx%dx%d (nz x ny x nx)" % shape), "bc": BC,

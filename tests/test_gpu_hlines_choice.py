@@ -96,3 +96,4 @@ def test_where_small_grids_take_them():
     assert _shapes((2, 1024, 4), "NNDDDD")["y-forward"] == Y[512]
     assert _shapes((2, 64, 4), "PPPPDD")["y-forward"] == Y[64]
     assert _shapes((2, 512, 4), "PPPPDD")["y-forward"] == Y[512]
+
