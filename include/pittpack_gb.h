@@ -71,7 +71,7 @@ typedef enum {
 typedef struct pp_plan_options {
   int threads_x;   /* CTA size of the x-line kernels (0 = automatic; FP64-class plans of large grids then take
                       block-scaled kernels of one fixed shape where y has 128 to 2048 = 2^a cells, or
-                      64 to 1024 = 2^a complex ones (2^19 cells on, some lengths from any size on), or x
+                      64 to 1024 = 2^a complex ones (0.5 to 1.3 M cells on, some lengths from any size on), or x
                       256 to 2048 = 2^a (12 M cells on), and the autotuner leaves those as they are) */
   int threads_y;   /* CTA size of the y-line kernels (0 = automatic) */
   int lines_x;     /* lines per CTA, x kernels (0 = automatic) */
