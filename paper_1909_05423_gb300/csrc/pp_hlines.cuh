@@ -211,7 +211,6 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
   const htwb* x1b = reinterpret_cast<const htwb*>(x1a + (M + 2));
   const htwa* x2a = reinterpret_cast<const htwa*>(x1b + (M + 2));
   const htwb* x2b = reinterpret_cast<const htwb*>(x2a + (M + 2));
-  pdl_start();
   for (int i = threadIdx.x; i < MC; i += H::T)
     cp_async_cx(reinterpret_cast<cx<df>*>(sta) + i, reinterpret_cast<const cx<df>*>(gta) + i);
   cp_async_commit();
@@ -358,6 +357,7 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
       stat(r[u][1]);
     }
     h_line_stats<OY, MC>(mx, l1, red, L);
+    pdl_start();
     S = hx_scale(a.hs, mx, l1);
 #pragma unroll
     for (int u = 0; u < 16; u++) v[u] = hcx{hx_from(r[u][0], S), hx_from(r[u][1], S)};
@@ -420,6 +420,7 @@ __global__ void __launch_bounds__((HShape<OY, MC>::T), (65536 / HRegs<HG, OY, MC
       hx_stat(mx, l1, rm[c].hi);
     }
     h_line_stats<OY, MC>(mx, l1, red, L);
+    pdl_start();
     S = hx_scale(a.hs, mx, l1);
     // E = X_k + conj X_{M-k}, O = (X_k - conj X_{M-k}) conj(w_N^k), both / 4; Z_k = E + i O, Z_{M-k} its
     // partner.  DCT-III / DST-III: X_k = A c, conj X_{M-k} = B c with A = Y_k - i Y_{N-k},

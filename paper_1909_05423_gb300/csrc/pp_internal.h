@@ -11,14 +11,17 @@
 namespace pp {
 
 // Programmatic dependent launch of the pipeline's kernels: a kernel's CTAs start as soon as every CTA of the
-// kernel before it has started and there is room, read what the plan holds (twiddles, mode descriptors) and
-// wait in pdl_wait() for that kernel to have finished and its writes to be visible.  Every kernel launched by
-// launch_pdl calls pdl_wait before it touches an array that another kernel writes or reads.  It hides launch
-// latency and prologues where a kernel is short: 32^3 alone 65.6 -> 58.9 us (back to back the host's launches
-// bound it), 120 x 140 x 99 167 -> 158 us.  Grids of more than 16 CTAs per SM are launched plainly: the CTAs
-// that start early hold room that the kernel before them still wants (256^3 535 -> 548 us, 1024^3 27.3 -> 30.5
-// ms).  So are the members of a batch graph, where other branches want that room (64 grids 2.88 -> 2.92 ms), and the
-// z sweeps (pp_zsolve.cu).
+// kernel before it has called pdl_start() (or ended) and there is room, read what the plan holds (twiddles, mode
+// descriptors) and wait in pdl_wait() for that kernel to have finished and its writes to be visible.  Every kernel
+// launched by launch_pdl calls pdl_wait before it touches an array that another kernel writes or reads, and
+// pdl_start where only its output is left to write (the block-scaled kernels, whose CTAs are longer, when a CTA has
+// read its input: before the output it cost the y kernels of type IV 8 %).  It hides launch latency and prologues
+// where a kernel is short: 32^3 49.0 -> 37.4 us back to back, 60.8 -> 53.0 alone; 399 grids of any shape 12 % on
+// average, single ones up to 6 % slower.  (With pdl_start at the top of the kernels, CTAs of two or three kernels
+// waited on the few SMs that had room and then ran there instead of one an SM: 45.8 us, 6 % on average, single grids up
+// to 20 % slower.)  Grids of more than 16 CTAs per SM are launched plainly (measured with the early start: 256^3
+// 535 -> 548 us, 1024^3 27.3 -> 30.5 ms).  So are the members of a batch graph, where other branches want that room (64
+// grids 2.88 -> 2.92 ms), and the z sweeps (pp_zsolve.cu).
 __device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 constexpr unsigned kPdlCtas = 16;  // CTAs per SM up to which launches overlap

@@ -912,7 +912,6 @@ __global__ void __maxnreg__((MaxRegs<R, MC, OY>::v)) k_lines(const LineArgs args
   long long* s_bin = reinterpret_cast<long long*>(tws + M);
   long long* s_bout = s_bin + a.lpc;
   const cx<R>* twg = reinterpret_cast<const cx<R>*>(a.tw);
-  pdl_start();
   // stage twiddles: w_M^j, j < M (run-time lengths) or the per-stage table of fft_lines_ct.
   // Asynchronous copies (cp.async), waited for after the pre-processing: their latency then
   // overlaps the line loads instead of preceding them.
@@ -958,6 +957,7 @@ __global__ void __maxnreg__((MaxRegs<R, MC, OY>::v)) k_lines(const LineArgs args
     else fft_lines<R, false, (MC < 0)>(buf, nl, ldm, a.fp, tws);
     if (a.fp.nst == 0) __syncthreads();
   }
+  pdl_start();
   post_tile<R, SO, OY, MCT>(a, buf, nl, s_bout);
 }
 

@@ -253,7 +253,6 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
   // of y_0, and c per line
   extern __shared__ float2 zp_sm[];
   float dmax = 0.0f, umax = 0.0f;
-  pdl_start();
   if ((int)blockIdx.x < a.nsing) {
     pdl_wait();
     zsing_block<S>(a, (int)blockIdx.x, zp_sm, dmax, umax);
@@ -399,6 +398,7 @@ __global__ void __launch_bounds__(ZpThreads<M>::v) k_zpart(const ZArgs a, int G,
   x = n1 ? zp_carry_near1(A, B, bA, bB, c, P, col, G, lgG, -1)
          : zp_carry<false>(A, B, bA, bB, c, P, col, G, lgG, -1, wide, terms);
   if (c == P - 1) x = top;
+  pdl_start();
   ZP_DISPATCH(zp_bwd2, v, x, R);
   if (live) {
     if (PER && k0 < qlen) {
